@@ -283,7 +283,8 @@ int mcd_get_total_rates(mcd_ctx *ctx, int32_t disk, double *Rtot, int32_t where)
 typedef struct {
     int32_t n_lo, n_hi;          /* particles per cell of the class's disks */
     int64_t cells;               /* cells in the class */
-    int32_t threads;             /* threads per cell */
+    int32_t threads;             /* threads per cell that own swarms or form rows (beside them the one-swarm-per-thread
+                                    variant runs a choice, a mass and a clock warp) */
     int32_t swarms_per_thread;   /* 1 or 2 (the control-warp variant: 1 per worker thread) */
     int32_t store;               /* dv matrix: 0 row i recomputed, 1 shared memory, 2 workspace */
     int32_t persistent;          /* persistent CTAs take cells by atomic ticket */

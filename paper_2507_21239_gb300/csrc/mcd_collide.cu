@@ -2,12 +2,15 @@
 // the largest-work-first queue, the cell classes and their launches, the
 // timed trial that picks each class's variant, and the probes.  The kernels
 // themselves are in mcd_collide.cuh, instantiated per (precision, swarms per
-// thread, exact total) in mcd_collide_f32s1.cu, mcd_collide_f32s2.cu,
-// mcd_collide_f32s1x.cu, mcd_collide_f32s2x.cu and mcd_collide_f64.cu, and the
-// control-warp variants in mcd_collide_ws.cuh (mcd_collide_f32ws4.cu,
-// mcd_collide_f32ws10.cu).
+// thread, exact total) in mcd_collide_f32s1.cu, mcd_collide_f32s2.cu, mcd_collide_f32s1x.cu,
+// mcd_collide_f32s2x.cu and mcd_collide_f64.cu, the mixed path's variants with
+// specialised warps (S = 1) in mcd_collide_chain.cuh
+// (mcd_collide_f32c2.cu, mcd_collide_f32c4.cu, mcd_collide_f32c8.cu,
+// mcd_collide_f32c16.cu), and the control-warp variants
+// in mcd_collide_ws.cuh (mcd_collide_f32ws4.cu, mcd_collide_f32ws10.cu).
 #include <algorithm>
 
+#include "mcd_collide_chain.cuh"
 #include "mcd_collide_ws.cuh"
 
 namespace mcd {
@@ -230,6 +233,21 @@ static cudaError_t variant(int op, int S, int store, bool ramp, bool tracer, boo
     }
 }
 
+// the chain variants for launches of nsl swarm slots
+static cudaError_t chain_variant(int op, int nsl, int store, bool ramp, bool tracer, unsigned grid, size_t smem,
+                                 cudaStream_t st, const CollideArgs *A, int *out)
+{
+    const int nthr = nsl + 32 * kChainRoles;
+    if (nsl <= 64)
+        return collide_chain_variant<4, kChainSmallCtas>(op, store, ramp, tracer, grid, nthr, smem, st, A, out);
+    switch (chain_slots(nsl)) {
+    case 4: return collide_chain_variant<4, 1>(op, store, ramp, tracer, grid, nthr, smem, st, A, out);
+    case 8: return collide_chain_variant<8, 1>(op, store, ramp, tracer, grid, nthr, smem, st, A, out);
+    case 16: return collide_chain_variant<16, 1>(op, store, ramp, tracer, grid, nthr, smem, st, A, out);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
 // the control-warp variants: swarms per control lane for cells of up to n
 // swarms (0: none fits)
 static int ws_pl(int n)
@@ -265,6 +283,7 @@ struct ClassLaunch {
     int S, store, nthr;
     size_t smem;
     int ws, pl;  // the control-warp variant and its swarms per control lane
+    int chain;   // the chain variant: nthr threads own swarms, and three more warps run beside them
 };
 
 // whether class k runs the control-warp variant: MCD_MIXED without the exact
@@ -287,6 +306,7 @@ static ClassLaunch class_launch(const CollideClass &k, int threads, int spt, int
     ClassLaunch L;
     L.ws = ws;
     L.pl = ws ? ws_pl(k.n_hi) : 0;
+    L.chain = 0;
     if (ws) {
         L.S = 1;
         L.store = usable_store<T>(k, dv_matrix >= 0 ? dv_matrix : k.store);
@@ -304,10 +324,20 @@ static ClassLaunch class_launch(const CollideClass &k, int threads, int spt, int
     if (sizeof(T) == 4 && !threads && block_threads<T>(class_threads(k.n_hi, 1), exact) > kMaxCell) L.S = 2;
     L.store = usable_store<T>(k, dv_matrix >= 0 ? dv_matrix : k.store);
     L.nthr = block_threads<T>(threads ? threads : class_threads(k.n_hi, L.S), exact);
-    L.smem = collide_smem_bytes<T>(L.nthr, L.S, tracer != 0, L.store, k.rows, k.W, exact);
+    L.chain = sizeof(T) == 4 && L.S == 1 && !exact;
+    auto bytes = [&]() {
+        return L.chain ? collide_chain_smem_bytes(L.nthr, tracer != 0, L.store, k.rows, k.W)
+                       : collide_smem_bytes<T>(L.nthr, L.S, tracer != 0, L.store, k.rows, k.W, exact);
+    };
+    L.smem = bytes();
+    if (L.chain && L.store == 1 && L.smem > (size_t)smem_optin) {  // (no room beside the ready outcomes)
+        L.chain = 0;
+        L.smem = bytes();
+    }
     if (L.store == 1 && L.smem > (size_t)smem_optin) {  // (the shared matrix no longer fits)
+        L.chain = sizeof(T) == 4 && L.S == 1 && !exact;
         L.store = usable_store<T>(k, 2);
-        L.smem = collide_smem_bytes<T>(L.nthr, L.S, tracer != 0, L.store, k.rows, k.W, exact);
+        L.smem = bytes();
     }
     // exclusive: request more than half an SM's shared memory so that no two
     // collide CTAs of classes that can carry long chains share an SM (the
@@ -337,6 +367,7 @@ template <class T>
 static cudaError_t launch_op(int op, const ClassLaunch &L, bool ramp, bool tracer, bool exact, unsigned grid,
                              cudaStream_t st, const CollideArgs *A, int *out)
 {
+    if (L.chain) return chain_variant(op, L.nthr, L.store, ramp, tracer, grid, L.smem, st, A, out);
     if (L.ws) return ws_variant(op, L.pl, L.store, ramp, tracer, grid, L.nthr, L.smem, st, A, out);
     return variant<T>(op, L.S, L.store, ramp, tracer, exact, grid, L.nthr, L.smem, st, A, out);
 }
@@ -410,6 +441,7 @@ static cudaError_t collide_impl(mcd_ctx *cx, int from_state, double t_end)
         A.n_queue = k.cells;
         A.dv_w = k.W;
         A.dv_rows = k.rows;
+        A.early = k.smem_fits;
         A.dvg = L.store == 2 ? k.dvg : nullptr;
         unsigned grid = (unsigned)k.cells;
         A.qhead = nullptr;
@@ -447,6 +479,7 @@ static cudaError_t prepare_impl(mcd_ctx *c)
         for (int S = 1; S <= (sizeof(T) == 4 ? 2 : 1); ++S)
             for (int store = 0; store <= 2; ++store) {
                 if (sizeof(T) == 8 && store == 1) continue;
+                if (sizeof(T) == 4 && S == 1 && !exact && store != 1) continue;  // (the chain variants, below)
                 int st = 0;
                 if ((e = variant<T>(2, S, store, false, false, exact, 0, 0, 0, nullptr, nullptr, &st)) != cudaSuccess)
                     return e;
@@ -454,6 +487,19 @@ static cudaError_t prepare_impl(mcd_ctx *c)
                 if (dyn <= 0) return cudaErrorInvalidValue;
                 if ((e = variant<T>(1, S, store, false, false, exact, 0, 0, (size_t)dyn, nullptr, nullptr,
                                     nullptr)) != cudaSuccess)
+                    return e;
+                smin = std::min(smin, dyn);
+            }
+    if (sizeof(T) == 4)
+        for (int nsl : {64, 128, 256, 512})
+            for (int store = 0; store <= 2; ++store) {
+                int st = 0;
+                if ((e = chain_variant(2, nsl, store, false, false, 0, 0, nullptr, nullptr, &st)) != cudaSuccess)
+                    return e;
+                const int dyn = optin - st;
+                if (dyn <= 0) return cudaErrorInvalidValue;
+                if ((e = chain_variant(1, nsl, store, false, false, 0, (size_t)dyn, nullptr, nullptr, nullptr)) !=
+                    cudaSuccess)
                     return e;
                 smin = std::min(smin, dyn);
             }
@@ -576,6 +622,7 @@ static cudaError_t tune_impl(mcd_ctx *c)
         A.n_queue = (int64_t)pick.size();
         A.dv_w = k.W;
         A.dv_rows = k.rows;
+        A.early = k.smem_fits;
         k.n_trials = 0;
         float best = 3.0e38f;
         for (const auto &cs : cand) {
@@ -583,7 +630,7 @@ static cudaError_t tune_impl(mcd_ctx *c)
                                                   c->exact_total, c->smem_optin, cs.ws);
             if (L.S != cs.S || L.store != cs.store) continue;  // (the launch would not run this candidate)
             if (L.smem > (size_t)c->smem_optin) continue;
-            A.dvg = L.store == 2 ? k.dvg : nullptr;
+                A.dvg = L.store == 2 ? k.dvg : nullptr;
             float ms[kTrialRuns + 1] = {};
             for (int rep = 0; rep <= kTrialRuns && e == cudaSuccess; ++rep) {
                 e = cudaMemcpyAsync(A.m, c->m[b], 8 * c->N, cudaMemcpyDeviceToDevice, st);

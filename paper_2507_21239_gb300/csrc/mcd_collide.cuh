@@ -54,10 +54,10 @@ namespace mcd {
 // ---- per-swarm cache -----------------------------------------------------------
 template <class T>
 struct alignas(16) Part {
-    T a, S, p, q;      // radius, Stokes number, 1/(1+S^2), 1/(1+S)
-    T im, mh, ml, ad;  // 1/m, mass as hi+lo, (a - a_sw) for Stokes-law swarms
-    T Mv, gi;          // M/V (times the cell's rate scale), 1/(dm m) (inf: no grouping)
-    T Sl;              // low part of S (FP32 path: S + Sl to ~2^-44)
+    T a, im, Mv, gi;   // radius, 1/m, M/V (times the cell's rate scale), 1/(dm m) (inf: no grouping):
+                       // what a rate needs beside a stored dv, one 16-byte load in FP32
+    T S, Sl, p, q;     // Stokes number and its low part (FP32 path: S + Sl to ~2^-44), 1/(1+S^2), 1/(1+S)
+    T mh, ml, ad;      // mass as hi+lo, (a - a_sw) for Stokes-law swarms
     int32_t fl;        // turbulence regime (0,1,2) | stokes << 2
 };
 
@@ -688,6 +688,7 @@ struct CollideArgs {
     unsigned long long *log_n;
     int64_t log_cap;
     int dv_w;         // row width of the stored matrix (STORE)
+    int early;        // chain variants: the class's matrix fits in shared memory (pair_flat)
     int dv_rows;      // rows per cell of the stored matrix (the class's largest cell)
     double *q;        // the tracer column (TRACER variants)
     void *dvg;        // STORE == 2: the class's matrices in the workspace, dv_rows x dv_w entries of T per queue entry
@@ -1091,22 +1092,14 @@ inline size_t collide_smem_bytes(int nthr, int S, bool tracer, int store, int ro
     return b;
 }
 
-// the variants' host entry points, one translation unit per (T, S, EXACT): op 0
-// launches the (store, ramp, tracer) variant; op 1 sets every ramp/tracer
-// variant of that store's dynamic shared-memory limit to `smem`; op 2 writes
-// the largest static shared memory of those variants to *out; op 3 writes the
-// variant's resident CTAs per SM at (nthr, smem) to *out
-template <class T, int S, bool EXACT>
-cudaError_t collide_variant(int op, int store, bool ramp, bool tracer, unsigned grid, int nthr, size_t smem,
-                            cudaStream_t st, const CollideArgs *A, int *out);
-
-template <class T, int S, int STORE, bool EXACT>
-cudaError_t collide_variant_store(int op, bool ramp, bool tracer, unsigned grid, int nthr, size_t smem,
-                                  cudaStream_t st, const CollideArgs *A, int *out)
+// one host operation on a store's four kernels (ks[(ramp ? 1 : 0) + (tracer ? 2 : 0)]): op 0
+// launches the (ramp, tracer) variant; op 1 sets every variant's dynamic
+// shared-memory limit to `smem`; op 2 writes the largest static shared memory
+// of the variants to *out; op 3 writes the variant's resident CTAs per SM at
+// (nthr, smem) to *out
+inline cudaError_t variant_op(void (*const ks[4])(CollideArgs), int op, bool ramp, bool tracer, unsigned grid,
+                              int nthr, size_t smem, cudaStream_t st, const CollideArgs *A, int *out)
 {
-    void (*ks[4])(CollideArgs) = {
-        k_collide<T, S, STORE, false, false, EXACT>, k_collide<T, S, STORE, true, false, EXACT>,
-        k_collide<T, S, STORE, false, true, EXACT>, k_collide<T, S, STORE, true, true, EXACT>};
     if (op == 0) {
         ks[(ramp ? 1 : 0) + (tracer ? 2 : 0)]<<<grid, nthr, smem, st>>>(*A);
         return cudaGetLastError();
@@ -1127,6 +1120,22 @@ cudaError_t collide_variant_store(int op, bool ramp, bool tracer, unsigned grid,
     }
     if (op == 2 && out) *out = mx;
     return e;
+}
+
+// the variants' host entry points, one translation unit per (T, S, EXACT);
+// ops as in variant_op
+template <class T, int S, bool EXACT>
+cudaError_t collide_variant(int op, int store, bool ramp, bool tracer, unsigned grid, int nthr, size_t smem,
+                            cudaStream_t st, const CollideArgs *A, int *out);
+
+template <class T, int S, int STORE, bool EXACT>
+cudaError_t collide_variant_store(int op, bool ramp, bool tracer, unsigned grid, int nthr, size_t smem,
+                                  cudaStream_t st, const CollideArgs *A, int *out)
+{
+    void (*ks[4])(CollideArgs) = {
+        k_collide<T, S, STORE, false, false, EXACT>, k_collide<T, S, STORE, true, false, EXACT>,
+        k_collide<T, S, STORE, false, true, EXACT>, k_collide<T, S, STORE, true, true, EXACT>};
+    return variant_op(ks, op, ramp, tracer, grid, nthr, smem, st, A, out);
 }
 
 }  // namespace mcd

@@ -1,7 +1,8 @@
-// mcd_collide_f32s1.cu -- the mixed-precision collide variants with 1 swarm per thread
-// (every dv-matrix store, with and without the fragmentation ramp and the
-// tracer), in a translation unit of their own so that the build compiles the
-// variants in parallel.
+// mcd_collide_f32s1.cu -- the mixed-precision block variant with one swarm per
+// thread and the shared-memory matrix (with and without the fragmentation ramp
+// and the tracer).  It runs where the chain variants' ready outcomes leave no
+// room for the matrix beside them (cells of about 290 to 318 swarms) and the
+// shared-memory matrix is asked for.
 #include "mcd_collide.cuh"
 
 namespace mcd {
@@ -10,12 +11,8 @@ template <>
 cudaError_t collide_variant<float, 1, false>(int op, int store, bool ramp, bool tracer, unsigned grid, int nthr,
                                         size_t smem, cudaStream_t st, const CollideArgs *A, int *out)
 {
-    switch (store) {
-    case 0: return collide_variant_store<float, 1, 0, false>(op, ramp, tracer, grid, nthr, smem, st, A, out);
-    case 1: return collide_variant_store<float, 1, 1, false>(op, ramp, tracer, grid, nthr, smem, st, A, out);
-    case 2: return collide_variant_store<float, 1, 2, false>(op, ramp, tracer, grid, nthr, smem, st, A, out);
-    default: return cudaErrorInvalidValue;
-    }
+    if (store != 1) return cudaErrorInvalidValue;
+    return collide_variant_store<float, 1, 1, false>(op, ramp, tracer, grid, nthr, smem, st, A, out);
 }
 
 }  // namespace mcd

@@ -393,24 +393,7 @@ cudaError_t collide_ws_variant_store(int op, bool ramp, bool tracer, unsigned gr
 {
     void (*ks[4])(CollideArgs) = {k_collide_ws<PL, STORE, false, false>, k_collide_ws<PL, STORE, true, false>,
                                   k_collide_ws<PL, STORE, false, true>, k_collide_ws<PL, STORE, true, true>};
-    if (op == 0) {
-        ks[(ramp ? 1 : 0) + (tracer ? 2 : 0)]<<<grid, nthr, smem, st>>>(*A);
-        return cudaGetLastError();
-    }
-    if (op == 3) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, ks[(ramp ? 1 : 0) + (tracer ? 2 : 0)], nthr, smem);
-    cudaError_t e = cudaSuccess;
-    int mx = 0;
-    for (int v = 0; v < 4 && e == cudaSuccess; ++v) {
-        if (op == 1) {
-            e = cudaFuncSetAttribute(ks[v], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        } else {
-            cudaFuncAttributes fa;
-            e = cudaFuncGetAttributes(&fa, ks[v]);
-            if (e == cudaSuccess && (int)fa.sharedSizeBytes > mx) mx = (int)fa.sharedSizeBytes;
-        }
-    }
-    if (op == 2 && out) *out = mx;
-    return e;
+    return variant_op(ks, op, ramp, tracer, grid, nthr, smem, st, A, out);
 }
 
 // host entry of the control-warp variants of one PL (same ops as

@@ -31,6 +31,9 @@ constexpr uint64_t kTagInit = 1, kTagCollide = 2, kTagTransport = 3;
 constexpr int kStNaN = 1, kStTimeout = 2, kStEmpty = 4, kStBadCell = 8;
 
 // ---- Philox4x64-10 (Salmon et al., SC'11) ---------------------------------
+constexpr uint64_t kPhiloxM0 = 0xD2E7470EE14C6C93ULL, kPhiloxM1 = 0xCA5A826395121157ULL;
+constexpr uint64_t kPhiloxW0 = 0x9E3779B97F4A7C15ULL, kPhiloxW1 = 0xBB67AE8584CAA73BULL;
+
 struct U4 {
     uint64_t x[4];
 };
@@ -50,20 +53,18 @@ __host__ __device__ inline void mulhilo(uint64_t a, uint64_t b, uint64_t &hi, ui
 __host__ __device__ inline U4 philox(uint64_t c0, uint64_t c1, uint64_t c2, uint64_t c3, uint64_t k0,
                                      uint64_t k1)
 {
-    const uint64_t M0 = 0xD2E7470EE14C6C93ULL, M1 = 0xCA5A826395121157ULL;
-    const uint64_t W0 = 0x9E3779B97F4A7C15ULL, W1 = 0xBB67AE8584CAA73BULL;
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
         uint64_t h0, l0, h1, l1;
-        mulhilo(M0, c0, h0, l0);
-        mulhilo(M1, c2, h1, l1);
+        mulhilo(kPhiloxM0, c0, h0, l0);
+        mulhilo(kPhiloxM1, c2, h1, l1);
         uint64_t n0 = h1 ^ c1 ^ k0, n2 = h0 ^ c3 ^ k1;
         c0 = n0;
         c1 = l1;
         c2 = n2;
         c3 = l0;
-        k0 += W0;
-        k1 += W1;
+        k0 += kPhiloxW0;
+        k1 += kPhiloxW1;
     }
     U4 o;
     o.x[0] = c0;
