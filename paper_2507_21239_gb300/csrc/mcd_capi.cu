@@ -82,6 +82,8 @@ size_t carve(mcd_ctx *c, void *base, Sizes &S, int32_t nd, int32_t prec)
     mcd_ctx *x = c ? c : &tmp;
     x->d_params = cv.take<mcd_disk_params>(nd);
     x->d_disks = cv.take<DiskDev>(nd);
+    x->d_cf = cv.take<DiskC<float>>(nd);
+    x->d_cd = cv.take<DiskC<double>>(nd);
     x->slot_disk = cv.take<int32_t>(S.N);
     x->cell_disk = cv.take<int32_t>(S.C);
     x->zone_disk = cv.take<int32_t>(S.Z);
@@ -299,6 +301,11 @@ int mcd_init_disk(mcd_ctx **out, const mcd_disk_params *p, const mcd_grid *g, in
     cp(c->queue_static, qstatic.data(), 4 * S.C);
     cp(c->d_params, p, sizeof(mcd_disk_params) * n_disks);
     cp(c->d_disks, S.disks.data(), sizeof(DiskDev) * n_disks);
+    std::vector<DiskC<float>> cf(n_disks);
+    std::vector<DiskC<double>> cd(n_disks);
+    for (int d = 0; d < n_disks; ++d) cf[d] = disk_consts<float>(p[d]), cd[d] = disk_consts<double>(p[d]);
+    cp(c->d_cf, cf.data(), sizeof(cf[0]) * n_disks);
+    cp(c->d_cd, cd.data(), sizeof(cd[0]) * n_disks);
     cp(c->cell_disk, cell_disk.data(), 4 * S.C);
     cp(c->zone_disk, zone_disk.data(), 4 * S.Z);
     cp(c->tile_disk, tile_disk.data(), 4 * S.T);

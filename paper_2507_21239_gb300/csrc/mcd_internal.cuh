@@ -137,13 +137,61 @@ __device__ inline float mlog(float x) { return logf(x); }
 __device__ inline double mexpm1(double x) { return expm1(x); }
 __device__ inline float mexpm1(float x) { return expm1f(x); }
 
-// all quantities of the static, vertically isothermal disk: power laws in r,
-// or log-log interpolation of the disk's gas table
+// What transport reads of a disk's parameters, as T: formed once per context
+// (disk_consts), because on GB300 every conversion from double runs on the FP64
+// unit (a warp instruction per ~19 SM cycles) and a particle would need a dozen.
 template <class T>
-__device__ inline Gas<T> gas_at(const mcd_disk_params &P, GasTab tab, double r, double z)
+struct DiskC {
+    T sigma0, p, T0, q, alpha, rho_s;
+    T mump, GM, lamc;           // mu m_p, G M_star, mu m_p / sigma_H2
+    double ca, r_in, r_out;     // ca = 3 / (4 pi rho_s): a^3 = ca m
+    float ca_h, ca_l;           // ca as a hi + lo pair
+    int32_t p2, q2;             // 2 p and 2 q where they are whole numbers from 0 to 8, else -1
+    int32_t moves, tr_flags, settle_form;  // moves: the disk has transport at all
+};
+template <class T>
+inline DiskC<T> disk_consts(const mcd_disk_params &P)
+{
+    DiskC<T> c;
+    c.sigma0 = (T)P.sigma0, c.p = (T)P.p, c.T0 = (T)P.T0, c.q = (T)P.q, c.alpha = (T)P.alpha, c.rho_s = (T)P.rho_s;
+    c.mump = (T)P.mu * (T)kMP;
+    c.GM = (T)(P.m_star * kGMsun);
+    c.lamc = c.mump / (T)P.sigma_h2;
+    c.ca = 3.0 / (4.0 * kPI * P.rho_s);
+    c.ca_h = (float)c.ca;
+    c.ca_l = (float)(c.ca - (double)c.ca_h);
+    c.r_in = P.r_in, c.r_out = P.r_out;
+    auto half = [](double x) {
+        for (int k = 0; k <= 8; ++k)
+            if (2.0 * x == (double)k) return k;
+        return -1;
+    };
+    c.p2 = half(P.p), c.q2 = half(P.q);
+    c.moves = P.kernel_mode != 1 && (P.tr_flags & (MCD_TR_RADIAL | MCD_TR_VERTICAL));
+    c.tr_flags = P.tr_flags;
+    c.settle_form = P.settle_form;
+    return c;
+}
+template <class T>
+__device__ __forceinline__ T gas_mump(const mcd_disk_params &P) { return (T)P.mu * (T)kMP; }
+template <class T>
+__device__ __forceinline__ T gas_GM(const mcd_disk_params &P) { return (T)(P.m_star * kGMsun); }
+template <class T>
+__device__ __forceinline__ T gas_lamc(const mcd_disk_params &P) { return (T)P.mu * (T)kMP / (T)P.sigma_h2; }
+template <class T>
+__device__ __forceinline__ T gas_mump(const DiskC<T> &P) { return P.mump; }
+template <class T>
+__device__ __forceinline__ T gas_GM(const DiskC<T> &P) { return P.GM; }
+template <class T>
+__device__ __forceinline__ T gas_lamc(const DiskC<T> &P) { return P.lamc; }
+
+// all quantities of the static, vertically isothermal disk: power laws in r,
+// or log-log interpolation of the disk's gas table.  rr, zz: r, z as T.  PT:
+// the disk's parameters, or DiskC<T> (the same bits).
+template <class T, class PT>
+__device__ inline Gas<T> gas_core(const PT &P, GasTab tab, double r, T rr, T zz)
 {
     Gas<T> g;
-    T rr = (T)r, zz = (T)z;
     if (tab.n >= 2) {
         const GasKnot &K = tab.k[gas_segment(tab, r)];
         if constexpr (sizeof(T) == 8) {
@@ -152,27 +200,27 @@ __device__ inline Gas<T> gas_at(const mcd_disk_params &P, GasTab tab, double r, 
             g.T_ = exp(K.lnT - K.q * dl);
         } else {
             // ln(r / r_k) from the ratio: exact to a few float ulps of a small number
-            const float dl = logf((float)r / (float)K.r);
+            const float dl = logf(rr / (float)K.r);
             g.Sigma = (float)K.S * expf(-(float)K.p * dl);
             g.T_ = (float)K.T * expf(-(float)K.q * dl);
         }
         g.p = (T)K.p;
         g.q = (T)K.q;
     } else {
-        T x = (T)r * (T)(1.0 / kAU);
+        T x = rr * (T)(1.0 / kAU);
         g.Sigma = (T)P.sigma0 * mpow(x, -(T)P.p);
         g.T_ = (T)P.T0 * mpow(x, -(T)P.q);
         g.p = (T)P.p;
         g.q = (T)P.q;
     }
-    g.cs = msqrt((T)kKB * g.T_ / ((T)P.mu * (T)kMP));
-    g.Omega = msqrt((T)(P.m_star * kGMsun) / rr / rr / rr);
+    g.cs = msqrt((T)kKB * g.T_ / gas_mump<T>(P));
+    g.Omega = msqrt(gas_GM<T>(P) / rr / rr / rr);
     g.H = g.cs / g.Omega;
     T rho_mid = g.Sigma / ((T)2.5066282746310002 * g.H);  // sqrt(2 pi)
     T s = zz / g.H;
     g.rho = rho_mid * mexp((T)-0.5 * s * s);
     g.vth = (T)1.5957691216057308 * g.cs;  // sqrt(8/pi)
-    g.lambda = ((T)P.mu * (T)kMP / (T)P.sigma_h2) / g.rho;
+    g.lambda = gas_lamc<T>(P) / g.rho;
     g.nu = (T)0.5 * g.vth * g.lambda;
     g.etavk = (T)0.5 * g.cs * g.cs / (g.Omega * rr) * (g.p + (T)0.5 * ((T)3 + g.q));
     g.D = (T)P.alpha * g.cs * g.H;
@@ -180,6 +228,12 @@ __device__ inline Gas<T> gas_at(const mcd_disk_params &P, GasTab tab, double r, 
     g.St_eta = (T)1 / msqrt(g.D / g.nu);
     g.asw = (T)2.25 * g.lambda;
     return g;
+}
+
+template <class T>
+__device__ inline Gas<T> gas_at(const mcd_disk_params &P, GasTab tab, double r, double z)
+{
+    return gas_core<T>(P, tab, r, (T)r, (T)z);
 }
 
 template <class T>
@@ -191,6 +245,27 @@ __device__ inline Gas<T> gas_at(const mcd_disk_params &P, double r, double z)
 __host__ __device__ inline double monomer_mass(const mcd_disk_params &P)
 {
     return P.m_init > 0.0 ? P.m_init : 4.0 * kPI / 3.0 * P.rho_s * P.a_mono * P.a_mono * P.a_mono;
+}
+
+// ---- conversions on the integer unit ------------------------------------------
+// (float)x and (double)f bit for bit without the FP64 unit, where the value is
+// zero-free and in range; the plain conversion otherwise (a branch that
+// particle data does not take)
+__device__ __forceinline__ float d2f_int(double x)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const unsigned lo = (unsigned)b, E = (unsigned)(b >> 52) & 0x7FFu;
+    if (E - 949u > 200u) return (float)x;
+    const unsigned up = ((lo >> 28) & 1u) & (((lo & 0x0FFFFFFFu) != 0u) | ((lo >> 29) & 1u));
+    const unsigned h = (unsigned)((b & 0x7FFFFFFFFFFFFFFFull) >> 29) - (896u << 23) + up;  // exponent rebiased mod 2^32
+    return __uint_as_float(h | ((unsigned)(b >> 32) & 0x80000000u));
+}
+__device__ __forceinline__ double f2d_int(float f)
+{
+    const unsigned x = __float_as_uint(f), a = x & 0x7FFFFFFFu;
+    if ((a >> 23) - 1u >= 254u) return (double)f;  // zero, subnormal, inf or NaN
+    return __longlong_as_double((long long)((((unsigned long long)a + (896ull << 23)) << 29) |
+                                            ((unsigned long long)(x & 0x80000000u) << 32)));
 }
 
 // ---- per-disk tables ---------------------------------------------------------
@@ -270,6 +345,8 @@ struct mcd_ctx {
     int64_t zone_max = 0, n0_max = 0;  // largest radial zone (n_z * per_cell) and disk (particles)
 
     mcd_disk_params *d_params = nullptr;
+    mcd::DiskC<float> *d_cf = nullptr;   // per disk: transport's constants (MCD_MIXED)
+    mcd::DiskC<double> *d_cd = nullptr;  // the same (MCD_FP64)
     mcd::DiskDev *d_disks = nullptr;
     int32_t *slot_disk = nullptr;  // disk of each particle slot [N]
     int32_t *cell_disk = nullptr;  // disk of each global cell [C]
