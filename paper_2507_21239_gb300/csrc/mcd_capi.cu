@@ -131,6 +131,7 @@ size_t carve(mcd_ctx *c, void *base, Sizes &S, int32_t nd, int32_t prec)
     x->diag_edges = cv.take<double>(MCD_MAX_BINS + 1);
     x->diag_out = cv.take<double>(5 * MCD_MAX_BINS);
     x->map_acc = cv.take<unsigned long long>(MCD_MAX_MAP_BINS + 1);
+    x->map_sums = cv.take<double>(kMapSums);
     x->map_redges = cv.take<double>(MCD_MAX_MAP_EDGES + 1);
     x->map_medges = cv.take<double>(MCD_MAX_MAP_EDGES + 1);
     x->map_out = cv.take<double>(MCD_MAX_MAP_BINS);

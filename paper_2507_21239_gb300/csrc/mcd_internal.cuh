@@ -307,6 +307,9 @@ constexpr int kCellKBytes = 384;
 // heavy chains of different classes run side by side.
 constexpr int kMaxClasses = 5;
 constexpr int kMaxTrials = 12;
+
+// warps of the sigma map's mass sum
+constexpr int kMapSums = 608 * 4;
 struct CollideClass {
     int32_t n_lo = 0, n_hi = 0;  // particles per cell of the class's disks
     int64_t cells = 0, qoff = 0; // its cells and their first queue position (class-major queue)
@@ -398,6 +401,7 @@ struct mcd_ctx {
     double *q[2] = {nullptr, nullptr};  // tracer column, double-buffered like the particle columns
     double *diag_edges = nullptr, *diag_out = nullptr;  // diagnostics: bin edges, per-bin sums
     unsigned long long *map_acc = nullptr;  // sigma map: per-bin unit counts, then the unit's exponent
+    double *map_sums = nullptr;  // sigma map: the warps' sums of the live mass
     double *map_redges = nullptr, *map_medges = nullptr, *map_out = nullptr;
     mcd::GasKnot *gas_knots = nullptr;  // [n_disks][MCD_MAX_GAS_KNOTS] gas tables
     int32_t *gas_n = nullptr;           // knots per disk (0: the power laws)
