@@ -25,9 +25,11 @@
 //    than dm m_i is absorbed, or erodes i, in groups of total mass dm m_i) are
 //    kept ready per swarm, new mass and swarm cache; other partners take the
 //    general outcome in the lane that found j.
-//  * while j is chosen the workers form the pair entries of one (SPEC = 1: the
-//    kind that came last) or both ready outcomes; if the event takes that
-//    outcome, its new row and column are there.
+//  * while j is chosen the workers form the new row and column of the ready
+//    outcome of the kind that came last, and (up to 256 swarms) the row sums they
+//    lead to; if the event takes that outcome, the next choice's prefixes follow
+//    at once.  Both ready outcomes together take longer than the choice: 100
+//    swarms 0.92 against 0.90 us per event.
 //  * the mass warp keeps the ready outcomes, masses and caches of the swarm that
 //    has just changed.
 //  * the clock warp sums the last event's new row (the fresh R_i), advances the
@@ -35,10 +37,11 @@
 //    one Philox round per event.
 //
 // Measured, heaviest cell, us per event (one thread per swarm with block-wide
-// scans before -> now): 50 swarms 1.35 -> 0.85, 100: 1.40 -> 0.93, 200: 1.53 ->
-// 1.03, 300: 1.69 -> 1.33, 400: 1.97 -> 1.49, 512: 2.01 -> 1.63.  Up to 256
-// swarms the shared matrix beats recomputing row i (200 swarms: 1.03 against
-// 1.13); where the ready outcomes leave no room for the matrix (from about 290)
+// scans before -> now): 50 swarms 1.35 -> 0.84, 100: 1.40 -> 0.90, 200: 1.53 ->
+// 0.98, 300: 1.69 -> 1.33, 400: 1.97 -> 1.48, 500: 2.01 -> 1.62.  (Without the
+// row sums formed ahead 0.93 at 100 and 1.03 at 200; with them 1.56 at 400,
+// where they compete with the choice for issue slots.)  Up to 256 swarms the
+// shared matrix beats recomputing row i (200 swarms: 0.98 against 1.14); where the ready outcomes leave no room for the matrix (from about 290)
 // recomputing in this layout beats the stored matrix in the block-scan layout
 // (1.33 against 1.69).  Two groups per worker warp, to issue what does not
 // depend on the swarm once per sub-partition, were slower at every size (200:
@@ -326,9 +329,9 @@ inline int chain_slots(int nsl) { return nsl <= 128 ? 4 : (nsl <= 256 ? 8 : 16);
 // row, the prefixes, dv of row i, and the stored matrix (STORE == 1)
 inline size_t collide_chain_smem_bytes(int nsl, bool tracer, int store, int rows, int W)
 {
-    size_t b = (size_t)nsl * (3 * sizeof(Part<float>) + 4 * sizeof(double) + (tracer ? sizeof(double) : 0) +
-                              (store == 1 ? 5 : 6) * sizeof(float)) +
-               sizeof(Part<float>) + 2 * sizeof(double) + 32 * chain_slots(nsl) * sizeof(float);
+    size_t b = (size_t)nsl * (3 * sizeof(Part<float>) + 6 * sizeof(double) + (tracer ? sizeof(double) : 0) +
+                              6 * sizeof(float)) +
+               sizeof(Part<float>) + sizeof(double2) + 32 * chain_slots(nsl) * sizeof(float);
     if (store == 1) b += (size_t)rows * W * sizeof(float);
     return b;
 }
@@ -383,21 +386,21 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
                                            ChainShared<NW> &sh, unsigned char *smem_raw)
 {
     typedef float T;
+    // the row sums a ready outcome leads to are formed ahead too, where the instructions fit
+    // into the time that the choice of j takes
+    constexpr bool AHEAD = NW <= 8 && MB == 1;
     constexpr int RW = 32 * NW;              // words of the posted new row
-    // (both for up to 128 swarms, where every sub-partition has one worker warp; with two or
-    // more the second one's instructions would outlast the choice of j)
-    constexpr int SPEC = NW == 4 && MB == 1 ? 2 : 1;    // ready outcomes whose pair entries are formed ahead
     const int nthr = blockDim.x, nsl = nthr - 32 * kChainRoles, ng = nsl >> 5;  // swarm slots (workers), groups
     Part<T> *parts = reinterpret_cast<Part<T> *>(smem_raw);
     Part<T> *ready = parts + nsl;  // [2][nsl]: grouped partner sticks, erodes; then a general outcome
     double2 *mm = reinterpret_cast<double2 *>(ready + 2 * nsl + 1);  // mass, dm m
-    double *mready = reinterpret_cast<double *>(mm + nsl);           // the masses of ready
-    double *qsh = mready + 2 * nsl + 2;                              // TRACER
+    double2 *mready = mm + nsl;                                      // the same of ready
+    double *qsh = reinterpret_cast<double *>(mready + 2 * nsl + 1);  // TRACER
     T *rn = reinterpret_cast<T *>(qsh + (TRACER ? nsl : 0));         // the last event's new row (zero beyond nsl)
     T *xs = rn + RW;                                                 // the scans' rows             
     T *pf = xs + 4 * nsl;                                      // prefixes within the groups
-    T *dvrow = pf + nsl;                                             // STORE != 1: dv of row i
-    T *Dm = dvrow;                                                   // STORE == 1
+    T *dvrow = pf + nsl;                                             // dv of row i
+    T *Dm = dvrow + nsl;                                             // STORE == 1
     const int W = A.dv_w;
     if constexpr (STORE == 2) Dm = reinterpret_cast<T *>(A.dvg) + (size_t)entry * A.dv_rows * W;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -450,7 +453,7 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
             const Part<T> pr = make_part_rn(c, mr, pk.Mv, kFlRenewed);
             if (act) {
                 ready[e * nsl + k] = pr;
-                mready[e * nsl + k] = mr;
+                mready[e * nsl + k] = make_double2(mr, __dmul_rn(c.dm, mr));
             }
         }
     }
@@ -492,6 +495,7 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
         const int gen = 2 * nsl;  // a general outcome's place among the ready ones
         int pend = -1;            // swarm whose fresh row sum rides on the next choice
         T vlo = (T)0, tot, tot2;
+        int64_t left = A.max_events;  // events before the cap
         if constexpr (RAMP) {  // the ramp's foot as the plain FP64 evaluation forms it
             const mcd_disk_params &P = A.params[disk];
             vlo = (T)(P.v_frag * (1.0 - P.frag_ramp));
@@ -503,9 +507,9 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
             bar_sync(kBarRates, nsl + 96);
             const T Rp = __int_as_float(sh.sel.y);
             const bool ihere = choose<NW>(sh.ti, pf, sh.at, dr.u1, pend, Rp, ng, n, tot, any, i, [](int) {});
-            if (!(tot > (T)0) || ev >= A.max_events) {  // (uniform)
+            if (!(tot > (T)0) || left <= 0) {  // (uniform)
                 if (lane == 0) {
-                    if (ev >= A.max_events && tot > (T)0 && !A.cap_stops) atomicOr(A.status, kStTimeout);
+                    if (left <= 0 && tot > (T)0 && !A.cap_stops) atomicOr(A.status, kStTimeout);
                     sh.pick.x = -2;
                     sh.sel.x = -2;
                 }
@@ -520,12 +524,13 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
             i = sh.sel.x;
             const double2 mmi = mm[i];
             const T Mvi = parts[i].Mv, mih = parts[i].mh;
-            double mj;
+            double mj, mst;
             T dvij;
             bar_sync(kBarRow, nsl + 32);
             const bool jhere = choose<NW>(sh.tj, pf, sh.at, dr.u2, -1, (T)0, ng, n, tot2, any, j, [&](int q) {
                 mj = mm[q].x;
-                dvij = STORE == 1 ? Dm[sym_at(i, q, n, W)] : dvrow[q];
+                dvij = dvrow[q];
+                mst = mmi.x + (dgt(mmi.y, mj) ? mmi.y : mj);  // should it stick (the FP64 latency behind the choice)
             });
             T dvx = dvij;
             if constexpr (RAMP)  // inside the ramp: fragments as at v_frag with the ramp's probability
@@ -538,12 +543,14 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
             if (any ? jhere : lane == 0) sh.pick.x = any ? (grouped ? (stick ? i : nsl + i) : gen) : -1;
             if (jhere && (!grouped || TRACER || logging)) {
                 if (!grouped) {
-                    if constexpr (RAMP)
+                    if (stick)
+                        mnew = mst;
+                    else if constexpr (RAMP)
                         mnew = outcome_ramp<T>(c, mmi.x, mj, mih, parts[j].mh, mmi.y, dvij, dr.u3, vlo, kind);
                     else
                         mnew = outcome<T>(c, mmi.x, mj, mih, parts[j].mh, mmi.y, dvij, dr.u3, kind);
                     ready[gen] = make_part_rn(c, mnew, Mvi, kFlRenewed);
-                    mready[gen] = mnew;
+                    mready[gen] = make_double2(mnew, __dmul_rn(c.dm, mnew));
                 } else {
                     mnew = ready_mass(c, mmi.x, mmi.y, !stick);  // (the mass warp may still be at work on mready)
                 }
@@ -573,6 +580,7 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
             }
             pend = i;
             ++ev;
+            --left;
             if (--until_rebuild == 0) {
                 pend = -1;
                 until_rebuild = reb;
@@ -596,8 +604,8 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
             // i's new mass and cache
             if (lane < 3) reinterpret_cast<uint4 *>(parts + i)[lane] = reinterpret_cast<const uint4 *>(ready + pick.x)[lane];
             const T Mvi = ready[pick.x].Mv;
-            const double mi = mready[pick.x], dmmi = __dmul_rn(c.dm, mi);
-            if (lane == 0) mm[i] = make_double2(mi, dmmi);
+            const double2 mi = mready[pick.x];
+            if (lane == 0) mm[i] = mi;
             __syncwarp();
             if (--until_rebuild == 0) {
                 bar_arrive(kBarBuild, nsl + 32);
@@ -605,13 +613,13 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
             }
             bar_arrive(kBarRates, nsl + 96);
             // its ready outcomes: even lanes stick, odd lanes erode
-            const double mnew = ready_mass(c, mi, dmmi, lane & 1);
+            const double mnew = ready_mass(c, mi.x, mi.y, lane & 1), dmnew = __dmul_rn(c.dm, mnew);
             __syncwarp();
             const Part<T> pnew = make_part_rn(c, mnew, Mvi, kFlRenewed);
             bar_sync(kBarRead, nsl + 32);
             if (lane < 2) {
                 ready[lane * nsl + i] = pnew;
-                mready[lane * nsl + i] = mnew;
+                mready[lane * nsl + i] = make_double2(mnew, dmnew);
             }
             __syncwarp();
             bar_arrive(kBarReady, nsl + 32);
@@ -657,7 +665,6 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
     } else {  // ---- the workers ----
         int pend = -1;  // swarm whose fresh row sum rides on the next choice
         Acc<T> R;
-        T colo = (T)0;
         // full build of the row sums: R_k = sum_j r_kj in j order, from the stored
         // matrix or from fresh entries two at a time
         auto build = [&]() {
@@ -683,28 +690,33 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
         build();
         bar_arrive(kBarNew, nsl + 32);
         T *const xw = xs + 128 * w;
-        int guess = 0;  // SPEC == 1: the kind of ready outcome that came last
+        int guess = 0;  // the kind of ready outcome that came last
+        // R_k for the next choice (0 for the swarm whose fresh sum rides on it), and
+        // what is put off until the choice is under way: the event's entry of the
+        // matrix, the updated R_k, and (took) the swarm's own new cache
+        T hi = act ? (T)R.hi() : (T)0, dvn = (T)0;
+        Acc<T> Rn = R;
+        Part<T> us = pk;
+        bool upd = false, took = false;
+        int at = 0;
         for (;;) {
             // (1) row sums for the choice of i: the previous event's R_i (the sum of
             //     its new row) is folded in there
-            T x = group_prefix(xw, (act && k != pend) ? (T)R.hi() : (T)0);
+            T x = group_prefix(xw, hi);
             pf[k] = x;
             if (lane == 31) sh.ti[2 * NW - ng + w] = x;
+            if (STORE != 0 && act && pend >= 0) Dm[at] = dvn;
             __syncwarp();
             bar_arrive(kBarRates, nsl + 96);
+            R.s = upd ? Rn.s : R.s;
+            R.c = upd ? Rn.c : R.c;
+            if (took) pk = us;  // (uniform)
             bar_sync(kBarI, nsl + 32);
             const int2 sel = sh.sel;
-            const int i = sel.x;
-            R.s = k == pend ? __int_as_float(sel.y) : R.s;
-            R.c = k == pend ? (T)0 : R.c;
-            if (i < 0) {
-                bar_sync(kBarReady, nsl + 32);
-                bar_sync(kBarEvent, nthr);
-                break;
-            }
+            const int i = max(sel.x, 0);
             // (2) row i (i meets k) and column i (k meets i) before the event
             const Part<T> pi = parts[i];
-            const int at = STORE != 0 ? sym_at(i, act ? k : n - 1, n, W) : 0;
+            at = STORE != 0 ? sym_at(i, act ? k : n - 1, n, W) : 0;
             T dvik, Kold;
             if constexpr (STORE != 0) {
                 dvik = Dm[at];
@@ -712,53 +724,78 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
             } else {
                 pair_flat1<true>(pc, early, pk, pi, dvik, Kold);
             }
-            if (STORE != 1) dvrow[k] = dvik;
-            colo = Kold * weight<T>(pk, pi);
+            R.s = k == pend ? __int_as_float(sel.y) : R.s;
+            R.c = k == pend ? (T)0 : R.c;
+            if (sel.x < 0) {
+                bar_sync(kBarReady, nsl + 32);
+                bar_sync(kBarEvent, nthr);
+                break;
+            }
+            dvrow[k] = dvik;
             x = group_prefix(xw, act ? Kold * weight<T>(pi, pk) : (T)0);
             pf[k] = x;
             if (lane == 31) sh.tj[2 * NW - ng + w] = x;
             __syncwarp();
             bar_arrive(kBarRow, nsl + 32);
-            // (3) meanwhile: the pair entries of the ready outcomes
+            const T colo = Kold * weight<T>(pk, pi);
+            // (3) meanwhile, for the ready outcome of the kind that came last: the new
+            //     row and column i, and the row sum they lead to
+            //     (R_k += r_ki(new) - r_ki(old))
             bar_sync(kBarReady, nsl + 32);
-            T dvs[SPEC], Ks[SPEC];
-            {
-                Part<T> u[SPEC], o[SPEC];
-#pragma unroll
-                for (int e = 0; e < SPEC; ++e) {
-                    o[e] = ready[(SPEC == 1 ? guess : e) * nsl + i];
-                    u[e] = part_select(k == i, o[e], pk);
-                }
-                pair_flat<SPEC, false>(pc, false, u, o, dvs, Ks);
+            upd = act && k != i;
+            const Part<T> o = ready[guess * nsl + i];
+            us = part_select(k == i, o, pk);
+            T dvs, Ks, rows, his;
+            Acc<T> Rs;
+            pair_flat1<false>(pc, false, us, o, dvs, Ks);
+            // (here, not where they are used: the compiler would sink them behind the barrier)
+            asm volatile("" : "+f"(Ks), "+f"(dvs));
+            if constexpr (AHEAD) {
+                rows = act ? Ks * weight<T>(o, us) : (T)0;
+                Rs = R;
+                Rs.update(Ks * weight<T>(us, o), colo);
+                his = upd ? (T)Rs.hi() : (T)0;
+                asm volatile("" : "+f"(rows), "+f"(his), "+f"(Rs.s), "+f"(Rs.c));
             }
             bar_sync(kBarEvent, nthr);
             const int2 pick = sh.pick;
             if (pick.x < 0 || pick.y) break;
-            // (4) new row and column i: R_k += r_ki(new) - r_ki(old); R_i afresh
+            // (4) the outcome's new row and column i: taken over, or formed now; R_i afresh
             const bool rebuild = --until_rebuild == 0;
-            const Part<T> pn = ready[pick.x];
-            const int kind = pick.x < nsl ? 0 : (pick.x < 2 * nsl ? 1 : 2);
-            pk = part_select(k == i, pn, pk);
-            T dvn = dvs[0], Knew = Ks[0];
-            if (SPEC == 2) dvn = kind ? dvs[SPEC - 1] : dvn, Knew = kind ? Ks[SPEC - 1] : Knew;
-            if (SPEC == 2 ? kind == 2 : kind != guess) pair_flat1<false>(pc, false, pk, pn, dvn, Knew);
-            guess = kind < 2 ? kind : guess;
-            if (STORE != 0 && act) Dm[at] = dvn;
-            rn[k] = (act && !rebuild) ? Knew * weight<T>(pn, pk) : (T)0;
-            __syncwarp();
-            bar_arrive(kBarNew, nsl + 32);
+            const bool hit = pick.x == guess * nsl + i;
+            took = AHEAD && hit;
+            dvn = dvs;
+            if (AHEAD && hit) {
+                hi = his;
+                rn[k] = rebuild ? (T)0 : rows;
+                __syncwarp();
+                bar_arrive(kBarNew, nsl + 32);
+                Rn = Rs;
+            } else {
+                const Part<T> pn = ready[pick.x];
+                T Knew = Ks;
+                pk = part_select(k == i, pn, pk);
+                if (!hit) pair_flat1<false>(pc, false, pk, pn, dvn, Knew);
+                rn[k] = act && !rebuild ? Knew * weight<T>(pn, pk) : (T)0;
+                __syncwarp();
+                bar_arrive(kBarNew, nsl + 32);
+                Rn = R;
+                Rn.update(Knew * weight<T>(pk, pn), colo);
+                hi = upd ? (T)Rn.hi() : (T)0;
+                guess = pick.x < nsl ? 0 : (pick.x < 2 * nsl ? 1 : guess);
+            }
             bar_arrive(kBarRead, nsl + 32);
-            Acc<T> Rn = R;
-            Rn.update(Knew * weight<T>(pk, pn), colo);
-            const bool upd = act && k != i;
-            R.s = upd ? Rn.s : R.s;
-            R.c = upd ? Rn.c : R.c;
             pend = i;
             if (rebuild) {
+                if (took) pk = us;
+                took = false;
+                if (STORE != 0 && act) Dm[at] = dvn;
                 bar_sync(kBarBuild, nsl + 32);
                 build();
+                Rn = R;
                 pend = -1;
                 until_rebuild = reb;
+                hi = act ? (T)R.hi() : (T)0;
             }
         }
         if (act) {
