@@ -178,6 +178,51 @@ __device__ __forceinline__ float lg2_mufu(float x)
     return y;
 }
 
+// ---- FP64 without the FP64 unit where that can be done ---------------------------
+// On GB300 an FP64 instruction of a warp holds its SM sub-partition's FP64 unit
+// for 64 cycles, whatever its lanes do, so the FP64 path counts those
+// instructions: comparisons, minima and conversions run on the integer unit,
+// reciprocals and square roots start from the FP32 special-function unit and
+// take one third-order step (Householder's iterations), three and five FP64
+// instructions, instead of the correctly rounded routines.  Values outside the
+// FP32 range take the plain operation (a branch that rates do not take).
+// A 0D cell of 200 swarms 9.5 -> 8.2 ms, 16 cells of 4 x 100 25.6 -> 21.4 ms a
+// step, 256 x 16 of 200 14.8 -> 11.0 ms; error of K against quadruple precision,
+// rms over the regimes, 1.92 -> 1.82e-16 (the correctly rounded routines round
+// more intermediate results).
+__device__ __forceinline__ bool in_f32_range(double x)
+{
+    return ((unsigned)(__double_as_longlong(x) >> 52) - 949u) <= 200u;  // positive, 2^-74 to 2^127
+}
+// 1 / b: with y good to 2^-22 and e = 1 - b y, y (1 + e + e^2) leaves e^3
+__device__ __forceinline__ double rcp64(double b)
+{
+    if (!in_f32_range(b)) return 1.0 / b;
+    float y0;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(d2f_int(b)));
+    const double y = f2d_int(y0), e = fma(-b, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+// sqrt(x): with y ~ 1/sqrt(x), t = x y and e = 1 - x y^2, t (1 + e/2 + 3 e^2/8) leaves e^3
+__device__ __forceinline__ double sqrt64(double x)
+{
+    if (!in_f32_range(x)) return sqrt(x);
+    float y0;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(d2f_int(x)));
+    const double y = f2d_int(y0), t = x * y, e = fma(-t, y, 1.0);
+    return fma(t, e * fma(0.375, e, 0.5), t);
+}
+// order of non-negative doubles through their bit patterns
+__device__ __forceinline__ double min_pos(double a, double b)
+{
+    return __double_as_longlong(a) < __double_as_longlong(b) ? a : b;
+}
+__device__ __forceinline__ double max_pos(double a, double b)
+{
+    return __double_as_longlong(a) < __double_as_longlong(b) ? b : a;
+}
+__device__ __forceinline__ float min_pos(float a, float b) { return fminf(a, b); }
+
 // (ah, al) < (bh, bl) for normalised hi + lo pairs
 __device__ __forceinline__ bool pair_lt(float ah, float al, float bh, float bl) { return ah < bh || (ah == bh && al < bl); }
 
@@ -189,19 +234,32 @@ template <>
 __device__ __forceinline__ Part<double> make_part<double>(const CellK<double> &c, double m, double Mv)
 {
     Part<double> q;
-    bool stk = m >= c.m_sw;
-    int cls = m < c.m_eta ? 0 : (m < c.m_one ? 1 : 2);
+    const long long mb = __double_as_longlong(m);  // (masses are positive)
+    const bool stk = mb >= __double_as_longlong(c.m_sw);
+    const int cls = mb < __double_as_longlong(c.m_eta) ? 0 : (mb < __double_as_longlong(c.m_one) ? 1 : 2);
     q.mh = m;
     q.ml = 0.0;
-    q.a = cbrt(c.cm_d * m);
+    const double x = c.cm_d * m;
+    if (in_f32_range(x)) {
+        // cbrt from FP32 (a0 to about 2^-21, 1/a0 alongside), then two Newton steps
+        // with the FP32 derivative: a error of 2^-21 goes to 2^-41 and 2^-61
+        const float l3 = lg2_mufu(d2f_int(x)) * (1.0f / 3.0f), ia = ex2_mufu(-l3);
+        const double h = f2d_int(ia * ia * (1.0f / 3.0f));
+        double a = f2d_int(ex2_mufu(l3));
+        a = fma(fma(-a * a, a, x), h, a);
+        a = fma(fma(-a * a, a, x), h, a);
+        q.a = a;
+    } else {
+        q.a = cbrt(x);
+    }
     q.S = stk ? c.Cst * q.a * q.a : c.Cep * q.a;
     q.Sl = 0.0;
-    q.p = 1.0 / (1.0 + q.S * q.S);
-    q.q = 1.0 / (1.0 + q.S);
-    q.im = 1.0 / m;
+    q.p = rcp64(fma(q.S, q.S, 1.0));
+    q.q = rcp64(1.0 + q.S);
+    q.im = rcp64(m);
     q.ad = stk ? c.cm_d * (m - c.m_sw) / ((q.a * q.a + c.asw * c.asw) + q.a * c.asw) : 0.0;
     q.Mv = Mv;
-    q.gi = c.dm > 0.0 ? 1.0 / (c.dm * m) : (double)INFINITY;
+    q.gi = c.dm > 0.0 ? rcp64(c.dm * m) : (double)INFINITY;
     q.fl = cls | ((int)stk << 2);
     return q;
 }
@@ -254,7 +312,7 @@ __device__ __forceinline__ Part<float> make_part<float>(const CellK<float> &c, d
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float fdiv(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double fdiv(double a, double b) { return a / b; }
+__device__ __forceinline__ double fdiv(double a, double b) { return a * rcp64(b); }
 
 // The constants one kernel entry reads; the FP32 path keeps them in registers
 // (read from shared memory at every entry they would sit on the critical path).
@@ -296,22 +354,21 @@ __device__ __forceinline__ T pair_dv(const C &c, const Part<T> &u, const Part<T>
         *K = c.Kc;
         return (T)0;
     }
-    // |St_u - St_v| from the factored difference of cubes
-    T dm = fabs((u.mh - v.mh) + (u.ml - v.ml));
-    T den = fma(u.a, v.a, mul_rn(u.a, u.a) + mul_rn(v.a, v.a));
-    T da = fdiv(c.cm * dm, den);
-    int su = u.fl >> 2, sv = v.fl >> 2;
-    T S1 = fmax(u.S, v.S), S2 = fmin(u.S, v.S);
-    int cls = max(u.fl & 3, v.fl & 3);
-    T D, tv;
-    if (sizeof(T) == 4) {
+    const int su = u.fl >> 2, sv = v.fl >> 2;
+    const int cls = max(u.fl & 3, v.fl & 3);
+    if constexpr (sizeof(T) == 4) {
         // FP32: every case evaluated and selected, so the lanes of a warp
         // never diverge (the regimes mix freely within a cell).  dv^2 is
         // factored as t0 + D^2 coef: everything but D (including the regime-I
         // division) is computed alongside D's own division.
+        // |St_u - St_v| from the factored difference of cubes
+        T dm = fabs((u.mh - v.mh) + (u.ml - v.ml));
+        T den = fma(u.a, v.a, mul_rn(u.a, u.a) + mul_rn(v.a, v.a));
+        T da = fdiv(c.cm * dm, den);
+        T S1 = fmax(u.S, v.S), S2 = fmin(u.S, v.S);
         T as = su ? u.a : v.a, ads = su ? u.ad : v.ad;
         T D_st = c.Cst * (u.a + v.a) * da, D_mx = c.Cst * fma(as, ads, c.asw * da), D_ep = c.Cep * da;
-        D = (su & sv) ? D_st : ((su | sv) ? D_mx : D_ep);
+        T D = (su & sv) ? D_st : ((su | sv) ? D_mx : D_ep);
         T s = S1 + S2;
         T g1 = fdiv(c.vg2 * fma(S1, S2, c.Se * s), s * (S1 + c.Se) * (S2 + c.Se));  // regime I: D^2 g1
         // regime II with eps = S2/S1 cleared from the fractions (one division):
@@ -332,48 +389,51 @@ __device__ __forceinline__ T pair_dv(const C &c, const Part<T> &u, const Part<T>
         *K = kern_of<T>(c, u.a, v.a, dv);
         return dv;
     } else {
-        if (su & sv) {
-            D = c.Cst * (u.a + v.a) * da;
-        } else if (su | sv) {
-            T as = su ? u.a : v.a, ads = su ? u.ad : v.ad;
-            D = c.Cst * fma(as, ads, c.asw * da);
-        } else {
-            D = c.Cep * da;
+        // FP64, about 46 FP64 instructions for the common case (two Epstein swarms,
+        // regime II) against some 150 with correctly rounded divisions and square
+        // root, and the warp's other regimes only where one of its lanes needs them.
+        const unsigned lanes = __activemask();
+        const T s2 = u.a + v.a;
+        const T da = c.cm * fabs(u.mh - v.mh) * rcp64(fma(s2, s2, -(u.a * v.a)));  // a_u - a_v from the cubes
+        T D = c.Cep * da;
+        if (__any_sync(lanes, su | sv)) {
+            const T as = su ? u.a : v.a, ads = su ? u.ad : v.ad;
+            D = (su & sv) ? c.Cst * s2 * da : ((su | sv) ? c.Cst * fma(as, ads, c.asw * da) : D);
         }
-        if (cls == 0) {
-            T s = S1 + S2;
-            tv = s > (T)0 ? fdiv(c.vg2 * D * D * fma(S1, S2, c.Se * s), s * (S1 + c.Se) * (S2 + c.Se)) : (T)0;
-        } else if (cls == 1) {
-            // vg2 S1 [2 y_a - (1+e) + 2/(1+e) (1/(1+y_a) + e^3/(y_a+e))], the last
-            // term over one common denominator
-            T eps = fdiv(S2, S1), ope = (T)1 + eps, yae = (T)kYA + eps;
-            T last = fdiv((T)2 * (yae * (T)(1.0 / (1.0 + kYA)) + eps * eps * eps), ope * yae);
-            tv = c.vg2 * S1 * (((T)(2.0 * kYA) - ope) + last);
-        } else {
-            tv = c.vg2 * (u.q + v.q);
+        const T S1 = max_pos(u.S, v.S), S2 = min_pos(u.S, v.S), s = S1 + S2, D2 = D * D;
+        T t0 = c.cbm * (u.im + v.im);
+        if (__double_as_longlong(c.vg2) > 0) {
+            if (__any_sync(lanes, cls == 1)) {
+                // regime II with eps = S2/S1 cleared from the fractions, as in FP32
+                const T A1 = fma((T)kYA, S1, S2);
+                const T num = fma(A1 * (S1 * S1), (T)(2.0 / (1.0 + kYA)), (T)2 * S2 * (S2 * S2));
+                const T t2 = fma(num, rcp64(s * A1), fma((T)(2.0 * kYA - 1.0), S1, -S2));
+                t0 = cls == 1 ? fma(c.vg2, t2, t0) : t0;
+            }
+            if (__any_sync(lanes, cls == 2)) t0 = cls == 2 ? fma(c.vg2, u.q + v.q, t0) : t0;
+            if (__any_sync(lanes, cls == 0)) {
+                const T g1 = c.vg2 * fma(S1, S2, c.Se * s) * rcp64(s * ((S1 + c.Se) * (S2 + c.Se)));
+                t0 = cls == 0 && __double_as_longlong(s) > 0 ? fma(D2, g1, t0) : t0;
+            }
         }
+        const T pp = u.p * v.p, om = fma(-u.S, v.S, (T)1);
+        T cz = c.oz2;
+        if (c.settle) {
+            const T qq = u.q * v.q;
+            cz *= qq * qq;
+        }
+        const T coef = fma(pp * pp, fma(c.e1 * s, s, c.e4 * om * om), cz);
+        const T dv = sqrt64(fma(D2, coef, t0));
+        *K = c.pi * s2 * s2 * dv;
+        return dv;
     }
-    T pp = u.p * v.p;
-    // 1 - S_u S_v with the product taken exactly and the low parts added
-    T om = fma(-u.S, v.S, (T)1) - (mul_rn(u.S, v.Sl) + mul_rn(u.Sl, v.S));
-    T sp = S1 + S2;
-    T D2 = D * D;
-    T rp = D2 * pp * pp * (c.e4 * om * om + c.e1 * sp * sp);
-    T sz = c.oz2 * D2;
-    if (c.settle) {
-        T qq = u.q * v.q;
-        sz *= qq * qq;
-    }
-    T dv = msqrt(c.cbm * (u.im + v.im) + tv + rp + sz);
-    *K = kern_of<T>(c, u.a, v.a, dv);
-    return dv;
 }
 
 // rate of swarm `self` meeting a particle of swarm `other`: K M_o/V min(1/m_o, 1/(dm m_self))
 template <class T>
 __device__ __forceinline__ T weight(const Part<T> &self, const Part<T> &other)
 {
-    return other.Mv * fmin(other.im, self.gi);
+    return other.Mv * min_pos(other.im, self.gi);
 }
 
 // ---- the cell's symmetric dv matrix in circulant half form ---------------------------
@@ -401,7 +461,15 @@ __device__ __forceinline__ int sym_at(int i, int j, int n, int W)
 // brackets the target and finds the thread by a ballot (and the element
 // within the thread from the previous thread's prefix).  block_bracket returns
 // the element in that warp's lane 0 and -1 in every other lane (one barrier).
-// A passive warp (no elements) skips its own scan.
+// A passive warp (no elements) skips its own scan.  FP64 comparisons go through
+// the bit patterns (prefixes of rates are not negative).
+__device__ __forceinline__ bool lt_rate(float a, float b) { return a < b; }
+__device__ __forceinline__ bool lt_rate(double a, double b) { return __double_as_longlong(a) < __double_as_longlong(b); }
+__device__ __forceinline__ bool finite_rate(float a) { return true; }  // (its comparisons see a NaN themselves)
+__device__ __forceinline__ bool finite_rate(double a)
+{
+    return ((unsigned)(__double_as_longlong(a) >> 52) & 0x7FFu) != 0x7FFu;
+}
 template <class V, int S, bool FUSE>
 __device__ __forceinline__ int block_bracket(const V (&x)[S], const V (&y)[S], V u, int pend, V *buf, V &total,
                                              V &ysum, bool passive = false)
@@ -445,12 +513,12 @@ __device__ __forceinline__ int block_bracket(const V (&x)[S], const V (&y)[S], V
     total = tot + Rp;
     ysum = Rp;
     V target = u * total;
-    if (target >= total) target = total * (V)(1.0 - 1e-7);
+    if (!lt_rate(target, total)) target = total * (V)(1.0 - 1e-7);
     const int e0 = S * (int)threadIdx.x;
     const V P = (off + wi) + ((pend >= 0 && e0 + S - 1 >= pend) ? Rp : (V)0);
     const V lo = off + ((pend >= 0 && S * 32 * w > pend) ? Rp : (V)0);
     const V hi = hib + ((pend >= 0 && S * 32 * (w + 1) - 1 >= pend) ? Rp : (V)0);
-    const unsigned bal = __ballot_sync(FULL, P > target);
+    const unsigned bal = __ballot_sync(FULL, lt_rate(target, P));
     // (a tree scan may leave lane 31's prefix an ulp below hi: then lane 31)
     const int l = __ffs(bal | 0x80000000u) - 1;
     int sub = 0;
@@ -472,7 +540,7 @@ __device__ __forceinline__ int block_bracket(const V (&x)[S], const V (&y)[S], V
         }
         sub = __shfl_sync(FULL, first >= 0 ? first : last, l);
     }
-    return (lane == 0 && lo <= target && target < hi) ? S * (32 * w + l) + sub : -1;
+    return (lane == 0 && finite_rate(total) && !lt_rate(target, lo) && lt_rate(target, hi)) ? S * (32 * w + l) + sub : -1;
 }
 
 // ---- compensated FP32 sums ---------------------------------------------------------
