@@ -100,7 +100,7 @@ size_t carve(mcd_ctx *c, void *base, Sizes &S, int32_t nd, int32_t prec)
     }
     int64_t H = 256 * S.T;
     x->hist = cv.take<uint32_t>(H);
-    x->scan_part = cv.take<uint32_t>(H / 4096 + 2);
+    x->sup = cv.take<uint32_t>((size_t)n_sup(S.T, S.disks.size()) * kRadixBins * kRadixUpperPasses);
     x->rfix_longs = cv.take<int64_t>(S.N / (kRunShortMax + 1) + 1);
     x->rfix_count = cv.take<int32_t>(2);
     x->cell_start = cv.take<int64_t>(S.C);
@@ -256,6 +256,7 @@ int mcd_init_disk(mcd_ctx **out, const mcd_disk_params *p, const mcd_grid *g, in
     c->C = S.C;
     c->Z = S.Z;
     c->n_tiles = S.T;
+    c->n_sup = n_sup(S.T, S.disks.size());
     c->n_max = S.n_max;
     for (int32_t d = 0; d < n_disks; ++d) {
         const int64_t zc = (int64_t)g[d].n_z * g[d].per_cell;

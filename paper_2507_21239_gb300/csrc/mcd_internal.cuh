@@ -286,10 +286,16 @@ struct StepState {
 // listed (so a list of N / (kRunShortMax + 1) + 1 entries always suffices)
 constexpr int kRunShortMax = 64;
 
-// radix sort tile: 256 threads x 16 keys
+// radix sort tile: 256 threads x 8 keys
 constexpr int kRadixThreads = 256, kRadixItems = 8, kRadixTile = kRadixThreads * kRadixItems;
 constexpr int kRadixBins = 256, kRadixPasses = 8;
+constexpr int kRadixGroup = 16;   // tiles per group (a disk's start at sup_off)
+constexpr int kRadixDirect = 64;  // groups a scatter CTA adds up itself
 constexpr int kRadixUpperPasses = 4;  // the r sort runs the passes of the keys' upper four bytes
+// A disk's first group: floor(t_off / 16) + its number leaves every disk room for
+// its last, partly filled group; n_sup is the end of the last disk's.
+__host__ __device__ constexpr int64_t n_sup(int64_t n_tiles, int64_t n_disks) { return n_tiles / kRadixGroup + n_disks; }
+__device__ __forceinline__ int64_t sup_off(const DiskDev &D, int64_t disk) { return D.t_off / kRadixGroup + disk; }
 
 // largest cell population the collide kernel takes (one thread per swarm)
 constexpr int kMaxCell = 512;
@@ -362,8 +368,9 @@ struct mcd_ctx {
 
     uint64_t *key[2] = {};
     uint32_t *val[2] = {};
-    uint32_t *hist = nullptr;      // [n_tiles * 256] in (disk, digit, tile) order
-    uint32_t *scan_part = nullptr; // block partials of the histogram scan
+    uint32_t *hist = nullptr;      // [n_tiles][256] digit counts of the current pass
+    uint32_t *sup = nullptr;       // [passes][n_sup][256] the groups' digit counts
+    int64_t n_sup = 0;             // groups of radix tiles, all disks
     int64_t *rfix_longs = nullptr; // the r sort's long runs of equal upper key words (first position each)
     int32_t *rfix_count = nullptr; // [0] long runs listed, [1] the fix-up CTAs' ticket
     int32_t n_sm_regrid = 0;       // SMs of the device (the long-run fix-up's grid)

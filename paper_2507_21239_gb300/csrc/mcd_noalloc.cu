@@ -27,7 +27,7 @@ namespace {
 
 constexpr int64_t kNoAllocMax = MCD_NOALLOC_MAX_PARTICLES;
 constexpr int64_t kTiles = (kNoAllocMax + mcd::kRadixTile - 1) / mcd::kRadixTile;
-constexpr int64_t kScanParts = (256 * kTiles) / 4096 + 2;
+constexpr int64_t kGroups = mcd::n_sup(kTiles, 1);
 
 // byte layout of the scratch array (each block 256-byte aligned)
 constexpr size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -41,8 +41,8 @@ constexpr size_t kOffKey1 = align256(kOffKey0 + 8 * kNoAllocMax);
 constexpr size_t kOffVal0 = align256(kOffKey1 + 8 * kNoAllocMax);
 constexpr size_t kOffVal1 = align256(kOffVal0 + 4 * kNoAllocMax);
 constexpr size_t kOffHist = align256(kOffVal1 + 4 * kNoAllocMax);
-constexpr size_t kOffPart = align256(kOffHist + 4 * 256 * kTiles);
-constexpr size_t kOffLongs = align256(kOffPart + 4 * kScanParts);
+constexpr size_t kOffSup = align256(kOffHist + 4 * 256 * kTiles);
+constexpr size_t kOffLongs = align256(kOffSup + 4 * 256 * kGroups * mcd::kRadixUpperPasses);
 constexpr size_t kOffRfix = align256(kOffLongs + 8 * (kNoAllocMax / (mcd::kRunShortMax + 1) + 1));
 constexpr size_t kOffAlive = align256(kOffRfix + 8);
 constexpr size_t kOffStatus = align256(kOffAlive + 8);
@@ -126,6 +126,7 @@ extern "C" int mcd_regrid_noalloc(const mcd_disk_params *p, const mcd_grid *g, c
     c.C = (int64_t)g->n_r * g->n_z;
     c.Z = g->n_r;
     c.n_tiles = D.n_tiles;
+    c.n_sup = mcd::n_sup(D.n_tiles, 1);
     c.n_max = g->per_cell;
     c.d_params = reinterpret_cast<mcd_disk_params *>(s + kOffParams);
     c.d_disks = reinterpret_cast<mcd::DiskDev *>(s + kOffDisk);
@@ -137,7 +138,7 @@ extern "C" int mcd_regrid_noalloc(const mcd_disk_params *p, const mcd_grid *g, c
     c.val[0] = reinterpret_cast<uint32_t *>(s + kOffVal0);
     c.val[1] = reinterpret_cast<uint32_t *>(s + kOffVal1);
     c.hist = reinterpret_cast<uint32_t *>(s + kOffHist);
-    c.scan_part = reinterpret_cast<uint32_t *>(s + kOffPart);
+    c.sup = reinterpret_cast<uint32_t *>(s + kOffSup);
     c.rfix_longs = reinterpret_cast<int64_t *>(s + kOffLongs);
     c.rfix_count = reinterpret_cast<int32_t *>(s + kOffRfix);
     c.n_alive = reinterpret_cast<int64_t *>(s + kOffAlive);

@@ -13,9 +13,15 @@
 //     position (disk offset + id), so a stable sort by r alone breaks ties by id;
 //  2. a segmented LSD radix sort of the keys' upper four bytes (sign, exponent
 //     and 20 mantissa bits), 4 passes of 8 bits, all disks in one launch
-//     sequence (tiles never straddle disks; the histogram is laid out disk-major,
-//     digit, tile so one exclusive scan yields every scatter offset), then every
-//     run of equal upper words put in (r, id) order (k_rfix, k_rfix_long);
+//     sequence, two launches per pass: a tile's digit counts, which are also added
+//     to its group's (16 tiles; tiles and groups never straddle disks), then the
+//     scatter, whose CTAs add up the groups and tiles before them themselves; then
+//     every run of equal upper words put in (r, id) order (k_rfix, k_rfix_long),
+//     and the removed particles moved along.  Up to a million particles a launch
+//     costs more than what it does, so 12 launches in place of 22 (a scan of all
+//     tiles' counts, two more launches a pass, the counters' clearing, a tail
+//     kernel) are what counts: a regrid of 65,536 particles 120 -> 85 us, of
+//     819,200 180 -> 146, of 1,638,400 280 -> 258, of 3,276,800 unchanged;
 //  3. one CTA per radial zone loads its (z, id) keys into shared memory, sorts
 //     them (radix on the upper words with the same run fix-up, or a bitonic
 //     network that needs no padding: every compare is ascending, absent
@@ -30,8 +36,8 @@ namespace mcd {
 
 __device__ __forceinline__ uint64_t order_key(double x)
 {
-    if (x == 0.0) x = 0.0;  // -0.0 -> +0.0
     uint64_t b = (uint64_t)__double_as_longlong(x);
+    if (!(b << 1)) b = 0;  // -0.0 -> +0.0 (integer unit: an FP64 comparison holds its sub-partition for 64 cycles)
     return (b & 0x8000000000000000ULL) ? ~b : (b | 0x8000000000000000ULL);
 }
 
@@ -41,16 +47,25 @@ __device__ __forceinline__ double key_value(uint64_t k)
     return __longlong_as_double((long long)b);
 }
 
+__device__ __forceinline__ bool is_nan(double x)
+{
+    return ((uint64_t)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFULL) > 0x7FF0000000000000ULL;
+}
+
 constexpr uint64_t kInfKey = 0xFFF0000000000000ULL;  // order_key(+inf)
 
+// the keys; and the groups' counts of every pass and the fix-up's counters cleared
 __global__ void k_regrid_keys(const DiskDev *disks, const int32_t *slot_disk, int64_t N, const double *r,
-                              const double *z, const uint32_t *id, uint64_t *key, uint32_t *val, int32_t *status)
+                              const double *z, const uint32_t *id, uint64_t *key, uint32_t *val, int32_t *status,
+                              uint32_t *sup, int64_t nsup, int32_t *rfix_count)
 {
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    for (int64_t q = s; q < nsup; q += (int64_t)gridDim.x * blockDim.x) sup[q] = 0;
+    if (s < 2) rfix_count[s] = 0;
     if (s >= N) return;
     int d = slot_disk[s];
     double rs = r[s];
-    if (isnan(rs) || isnan(z[s])) {
+    if (is_nan(rs) || is_nan(z[s])) {
         atomicOr(status, kStNaN);
         rs = INFINITY;
     }
@@ -80,14 +95,10 @@ __device__ __forceinline__ unsigned digit_peers(int digit, bool ok)
     return ok ? peers : 0u;
 }
 
-// histogram index of (tile t of disk d, digit b)
-__device__ __forceinline__ int64_t hidx(const DiskDev &D, int64_t t, int b)
-{
-    return 256 * D.t_off + (int64_t)b * D.n_tiles + (t - D.t_off);
-}
-
+// tile t's digit counts to hist[t][.], and added to its group's, sup[group][.]
 __global__ void __launch_bounds__(kRadixThreads) k_radix_hist(const DiskDev *disks, const int32_t *tile_disk,
-                                                              const uint64_t *key, int shift, uint32_t *hist)
+                                                              const uint64_t *key, int shift, uint32_t *hist,
+                                                              uint32_t *sup)
 {
     __shared__ uint32_t h[kRadixBins];
     int64_t t = blockIdx.x;
@@ -98,14 +109,15 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_hist(const DiskDev *dis
     __syncthreads();
     for (int64_t q = start + threadIdx.x; q < end; q += kRadixThreads) atomicAdd(&h[(key[q] >> shift) & 255], 1u);
     __syncthreads();
-    hist[hidx(D, t, threadIdx.x)] = h[threadIdx.x];
+    const uint32_t x = h[threadIdx.x];
+    hist[t * kRadixBins + threadIdx.x] = x;
+    if (x) atomicAdd(&sup[(sup_off(D, tile_disk[t]) + (t - D.t_off) / kRadixGroup) * kRadixBins + threadIdx.x], x);
 }
 
-constexpr int kScanThreads = 1024, kScanItems = 4, kScanBlock = kScanThreads * kScanItems;
-
-__device__ __forceinline__ uint32_t block_excl_scan_u32(uint32_t x, uint32_t *wsum, uint32_t &total)
+// exclusive scan of one value per thread over the 256 digits of a block
+__device__ __forceinline__ uint32_t digit_excl_scan(uint32_t x, uint32_t *wsum)
 {
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     uint32_t v = x;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -114,54 +126,49 @@ __device__ __forceinline__ uint32_t block_excl_scan_u32(uint32_t x, uint32_t *ws
     }
     if (lane == 31) wsum[w] = v;
     __syncthreads();
-    if (w == 0) {
-        uint32_t s = lane < nw ? wsum[lane] : 0;
+    uint32_t off = 0;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            uint32_t y = __shfl_up_sync(0xffffffffu, s, o);
-            if (lane >= o) s += y;
-        }
-        if (lane < nw) wsum[lane] = s;
-    }
+    for (int ww = 0; ww < kRadixThreads / 32; ++ww) off += ww < w ? wsum[ww] : 0u;
     __syncthreads();
-    total = wsum[nw - 1];
-    uint32_t res = v - x + (w > 0 ? wsum[w - 1] : 0);
-    __syncthreads();
-    return res;
+    return off + v - x;
 }
 
-// exclusive scan of each block of kScanBlock entries in place; block totals to part
-__global__ void __launch_bounds__(kScanThreads) k_scan_blocks(uint32_t *a, int64_t n, uint32_t *part)
-{
-    __shared__ uint32_t wsum[32];
-    int64_t base = blockIdx.x * (int64_t)kScanBlock + threadIdx.x * kScanItems;
-    uint32_t v[kScanItems], s = 0;
-#pragma unroll
-    for (int i = 0; i < kScanItems; ++i) {
-        v[i] = base + i < n ? a[base + i] : 0;
-        s += v[i];
-    }
-    uint32_t tot;
-    uint32_t ex = block_excl_scan_u32(s, wsum, tot);
-#pragma unroll
-    for (int i = 0; i < kScanItems; ++i) {
-        if (base + i < n) a[base + i] = ex;
-        ex += v[i];
-    }
-    if (threadIdx.x == 0) part[blockIdx.x] = tot;
-}
+// Large disks: one CTA per disk turns the groups' counts into their first
+// destination per digit, so that a scatter CTA reads one row instead of all.
+// Up to kRadixDirect groups (2,097,152 particles) a CTA adds them up itself, a
+// launch less per pass; a regrid added up / scanned: 65,536 particles 85 / 101
+// us, 819,200 146 / 156, 1,638,400 (50 groups) 258 / 270, 3,276,800 (100
+// groups) 790 / 767.
+constexpr int kSupSlices = 4;  // a disk's groups in four slices: the loads are what it waits for
 
-// exclusive scan of the block totals (one CTA, any length)
-__global__ void __launch_bounds__(kScanThreads) k_scan_parts(uint32_t *part, int64_t n)
+__global__ void __launch_bounds__(kSupSlices *kRadixBins) k_sup_scan(const DiskDev *disks, uint32_t *sup)
 {
-    __shared__ uint32_t wsum[32];
-    uint32_t carry = 0;
-    for (int64_t base = 0; base < n; base += kScanThreads) {
-        int64_t q = base + threadIdx.x;
-        uint32_t x = q < n ? part[q] : 0, tot;
-        uint32_t ex = block_excl_scan_u32(x, wsum, tot);
-        if (q < n) part[q] = ex + carry;
-        carry += tot;
+    __shared__ uint32_t part[kSupSlices][kRadixBins], first[kRadixBins], wsum[32];
+    const DiskDev D = disks[blockIdx.x];
+    const int b = threadIdx.x & (kRadixBins - 1), j = threadIdx.x / kRadixBins;
+    const int64_t ns = (D.n_tiles + kRadixGroup - 1) / kRadixGroup;
+    const int64_t g0 = ns * j / kSupSlices, g1 = ns * (j + 1) / kSupSlices;
+    uint32_t *row = sup + sup_off(D, blockIdx.x) * kRadixBins + b;
+    uint32_t tot = 0;
+#pragma unroll 16
+    for (int64_t g = g0; g < g1; ++g) tot += row[g * kRadixBins];
+    part[j][b] = tot;
+    __syncthreads();
+    uint32_t dtot = 0, before = 0;
+    for (int q = 0; q < kSupSlices; ++q) {
+        dtot += part[q][b];
+        before += q < j ? part[q][b] : 0u;
+    }
+    // (of the slices, the first's eight warps hold the scan over the digits)
+    const uint32_t x = digit_excl_scan(dtot, wsum);
+    if (j == 0) first[b] = x;
+    __syncthreads();
+    uint32_t run = first[b] + before;
+#pragma unroll 16
+    for (int64_t g = g0; g < g1; ++g) {
+        const uint32_t x = row[g * kRadixBins];
+        row[g * kRadixBins] = run;
+        run += x;
     }
 }
 
@@ -176,7 +183,7 @@ constexpr size_t kScatterStage = (size_t)kRadixTile * (sizeof(uint64_t) + sizeof
 __global__ void __launch_bounds__(kRadixThreads, 4) k_radix_scatter(const DiskDev *disks, const int32_t *tile_disk,
                                                                  const uint64_t *ksrc, const uint32_t *vsrc,
                                                                  uint64_t *kdst, uint32_t *vdst, int shift,
-                                                                 const uint32_t *hist, const uint32_t *part)
+                                                                 const uint32_t *hist, const uint32_t *sup, int scanned)
 {
     __shared__ uint32_t wcnt[kRadixThreads / 32][kRadixBins];
     __shared__ uint32_t toff[kRadixBins], loff[kRadixBins], wsum[32];
@@ -189,9 +196,26 @@ __global__ void __launch_bounds__(kRadixThreads, 4) k_radix_scatter(const DiskDe
     int64_t start = D.p_off + (t - D.t_off) * kRadixTile;
     int64_t end = min(start + kRadixTile, D.p_off + D.n0);
     const int nvalid = (int)(end - start);
+    // the digits' first destinations: the counts of the tiles of this group before
+    // this one, and of the groups before it behind the smaller digits' totals
+    uint32_t before = 0, dtot = 0;
     {
-        int64_t hi = hidx(D, t, threadIdx.x);
-        toff[threadIdx.x] = hist[hi] + part[hi / kScanBlock];
+        const int64_t lt = t - D.t_off, g = lt / kRadixGroup;
+        const uint32_t *row = sup + sup_off(D, tile_disk[t]) * kRadixBins + threadIdx.x;
+        if (scanned) {
+            before = row[g * kRadixBins];
+        } else {
+            const int ns = (int)((D.n_tiles + kRadixGroup - 1) / kRadixGroup);
+#pragma unroll 8
+            for (int q = 0; q < ns; ++q) {
+                const uint32_t x = row[q * kRadixBins];
+                dtot += x;
+                before += q < g ? x : 0u;
+            }
+        }
+        const uint32_t *hrow = hist + threadIdx.x;
+#pragma unroll 8
+        for (int64_t q = D.t_off + g * kRadixGroup; q < t; ++q) before += hrow[q * kRadixBins];
     }
     for (int q = threadIdx.x; q < (kRadixThreads / 32) * kRadixBins; q += kRadixThreads) (&wcnt[0][0])[q] = 0;
     // every load of the tile issued before the first use
@@ -205,6 +229,7 @@ __global__ void __launch_bounds__(kRadixThreads, 4) k_radix_scatter(const DiskDe
         kk[it] = ok ? ksrc[start + lq] : 0;
         vv[it] = ok ? vsrc[start + lq] : 0;
     }
+    toff[threadIdx.x] = (uint32_t)D.p_off + before + (scanned ? 0u : digit_excl_scan(dtot, wsum));
     __syncthreads();
     const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
@@ -239,20 +264,7 @@ __global__ void __launch_bounds__(kRadixThreads, 4) k_radix_scatter(const DiskDe
         cnt = run;
     }
     // exclusive scan of the digit counts: the digit's first slot in the staged tile
-    {
-        uint32_t v = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            uint32_t y = __shfl_up_sync(0xffffffffu, v, o);
-            if (lane >= o) v += y;
-        }
-        if (lane == 31) wsum[w] = v;
-        __syncthreads();
-        uint32_t off = 0;
-#pragma unroll
-        for (int ww = 0; ww < kRadixThreads / 32; ++ww) off += ww < w ? wsum[ww] : 0u;
-        loff[threadIdx.x] = off + v - cnt;
-    }
+    loff[threadIdx.x] = digit_excl_scan(cnt, wsum);
     __syncthreads();
 #pragma unroll
     for (int it = 0; it < kRadixItems; ++it) {
@@ -344,8 +356,18 @@ constexpr int kZoneThreads = 512;  // two zones per SM
 // already in order.
 constexpr int kRunShort = kRunShortMax;
 
+// the particle columns from one buffer to the other (q: the tracer's, or null)
+struct Columns {
+    const double *m0, *M0, *r0, *z0;
+    const uint32_t *id0;
+    double *m1, *M1, *r1, *z1;
+    uint32_t *id1;
+    const double *q0;
+    double *q1;
+};
+
 __global__ void k_rfix(const DiskDev *disks, const int32_t *slot_disk, int64_t N, uint64_t *key, uint32_t *val,
-                       int64_t *longs, int32_t *n_long, int64_t *n_alive, int32_t *status)
+                       int64_t *longs, int32_t *n_long, int64_t *n_alive, int32_t *status, Columns A)
 {
     const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (s >= N) return;
@@ -359,6 +381,16 @@ __global__ void k_rfix(const DiskDev *disks, const int32_t *slot_disk, int64_t N
     if (!fin && s == D.p_off) {
         n_alive[d] = 0;
         atomicOr(status, kStEmpty);
+    }
+    if (!fin) {  // a removed particle keeps its place at the disk's tail, in id order
+        const int64_t gs = D.p_off + ((int64_t)val[s] < D.n0 ? val[s] : 0);
+        A.m1[s] = A.m0[gs];
+        A.M1[s] = A.M0[gs];
+        A.r1[s] = A.r0[gs];
+        A.z1[s] = A.z0[gs];
+        A.id1[s] = A.id0[gs];
+        if (A.q0) A.q1[s] = A.q0[gs];
+        return;
     }
     const uint32_t hi = (uint32_t)(key[s] >> 32);
     if (hi == (uint32_t)(kInfKey >> 32)) return;
@@ -576,12 +608,7 @@ struct ZoneArgs {
     const int64_t *n_alive;
     const uint64_t *rkey;  // sorted r keys
     const uint32_t *rsrc;  // disk-local source slot of each sorted position
-    const double *m0, *M0, *r0, *z0;
-    const uint32_t *id0;
-    double *m1, *M1, *r1, *z1;
-    uint32_t *id1;
-    const double *q0;  // the tracer column, or null
-    double *q1;
+    Columns col;
     int64_t *cell_start;
     int32_t *cell_n;
     double *cell_b, *cell_V;
@@ -618,13 +645,13 @@ __global__ void __launch_bounds__(kZoneThreads, 2) k_zone(ZoneArgs A)
                 src = 0;
             }
             int64_t gs = D.p_off + src;
-            double zz = A.z0[gs];
-            if (isnan(zz)) {
+            double zz = A.col.z0[gs];
+            if (is_nan(zz)) {
                 atomicOr(A.status, kStNaN);
                 zz = INFINITY;
             }
             const uint64_t kz = order_key(zz);
-            el[q] = make_uint4((uint32_t)kz, (uint32_t)(kz >> 32), A.id0[gs], src);
+            el[q] = make_uint4((uint32_t)kz, (uint32_t)(kz >> 32), A.col.id0[gs], src);
         }
         __syncthreads();
     };
@@ -739,33 +766,13 @@ __global__ void __launch_bounds__(kZoneThreads, 2) k_zone(ZoneArgs A)
     for (int64_t q = threadIdx.x; q < nk; q += blockDim.x) {
         const uint4 e = el[q];
         int64_t gs = D.p_off + e.w, gd = D.p_off + zs + q;
-        A.m1[gd] = A.m0[gs];
-        A.M1[gd] = A.M0[gs];
-        A.r1[gd] = A.r0[gs];
-        A.z1[gd] = key_value(el_key(e));
-        A.id1[gd] = e.z;
-        if (A.q0) A.q1[gd] = A.q0[gs];
+        A.col.m1[gd] = A.col.m0[gs];
+        A.col.M1[gd] = A.col.M0[gs];
+        A.col.r1[gd] = A.col.r0[gs];
+        A.col.z1[gd] = key_value(el_key(e));
+        A.col.id1[gd] = e.z;
+        if (A.col.q0) A.col.q1[gd] = A.col.q0[gs];
     }
-}
-
-// removed particles: sorted positions [n_alive, n0) of each disk, in id order
-__global__ void k_dead_tail(const DiskDev *disks, const int32_t *slot_disk, int64_t N, const int64_t *n_alive,
-                            const uint32_t *rsrc, const double *m0, const double *M0, const double *r0,
-                            const double *z0, const uint32_t *id0, double *m1, double *M1, double *r1, double *z1,
-                            uint32_t *id1, const double *q0, double *q1)
-{
-    int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (s >= N) return;
-    int d = slot_disk[s];
-    const DiskDev D = disks[d];
-    if (s - D.p_off < n_alive[d]) return;
-    int64_t gs = D.p_off + ((int64_t)rsrc[s] < D.n0 ? rsrc[s] : 0);
-    m1[s] = m0[gs];
-    M1[s] = M0[gs];
-    r1[s] = r0[gs];
-    z1[s] = z0[gs];
-    id1[s] = id0[gs];
-    if (q0) q1[s] = q0[gs];
 }
 
 // the zone sort: the largest zone's size, the path (radix when the zone fits
@@ -811,26 +818,29 @@ cudaError_t launch_regrid(mcd_ctx *c)
     cudaStream_t st = c->stream;
     const int b = c->cur, nb = 1 - c->cur;
     unsigned gN = (unsigned)((c->N + 255) / 256);
+    const int64_t nsup = c->n_sup * kRadixBins;
     k_regrid_keys<<<gN, 256, 0, st>>>(c->d_disks, c->slot_disk, c->N, c->r[b], c->z[b], c->id[b], c->key[0],
-                                      c->val[0], c->status);
-    const int64_t H = 256 * c->n_tiles;
-    const unsigned nsb = (unsigned)((H + kScanBlock - 1) / kScanBlock);
+                                      c->val[0], c->status, c->sup, nsup * kRadixUpperPasses, c->rfix_count);
+    const int64_t groups_max = (c->n0_max + (int64_t)kRadixTile * kRadixGroup - 1) / ((int64_t)kRadixTile * kRadixGroup);
+    const int scanned = groups_max > kRadixDirect;
     // the upper four bytes of the keys (an even number of passes: the result is back in buffer 0)
     for (int pass = kRadixPasses - kRadixUpperPasses; pass < kRadixPasses; ++pass) {
         const int shift = 8 * pass, src = pass & 1, dst = src ^ 1;
+        uint32_t *sup = c->sup + nsup * (pass - (kRadixPasses - kRadixUpperPasses));
         k_radix_hist<<<(unsigned)c->n_tiles, kRadixThreads, 0, st>>>(c->d_disks, c->tile_disk, c->key[src], shift,
-                                                                     c->hist);
-        k_scan_blocks<<<nsb, kScanThreads, 0, st>>>(c->hist, H, c->scan_part);
-        k_scan_parts<<<1, kScanThreads, 0, st>>>(c->scan_part, nsb);
+                                                                     c->hist, sup);
+        if (scanned) k_sup_scan<<<(unsigned)c->n_disks, kSupSlices * kRadixBins, 0, st>>>(c->d_disks, sup);
         k_radix_scatter<<<(unsigned)c->n_tiles, kRadixThreads, kScatterStage, st>>>(
-            c->d_disks, c->tile_disk, c->key[src], c->val[src], c->key[dst], c->val[dst], shift, c->hist,
-            c->scan_part);
+            c->d_disks, c->tile_disk, c->key[src], c->val[src], c->key[dst], c->val[dst], shift, c->hist, sup, scanned);
     }
-    // runs of equal upper words into (key, id) order
-    cudaError_t e = cudaMemsetAsync(c->rfix_count, 0, 2 * sizeof(int32_t), st);
-    if (e != cudaSuccess) return e;
+    Columns col;
+    col.m0 = c->m[b]; col.M0 = c->M[b]; col.r0 = c->r[b]; col.z0 = c->z[b]; col.id0 = c->id[b];
+    col.m1 = c->m[nb]; col.M1 = c->M[nb]; col.r1 = c->r[nb]; col.z1 = c->z[nb]; col.id1 = c->id[nb];
+    col.q0 = c->tracer ? c->q[b] : nullptr;
+    col.q1 = c->tracer ? c->q[nb] : nullptr;
+    // runs of equal upper words into (key, id) order; removed particles to the tail
     k_rfix<<<gN, 256, 0, st>>>(c->d_disks, c->slot_disk, c->N, c->key[0], c->val[0], c->rfix_longs, c->rfix_count,
-                               c->n_alive, c->status);
+                               c->n_alive, c->status, col);
     k_rfix_long<<<(unsigned)std::max(1, std::min(c->n_sm_regrid, 1024)), kZoneThreads, kZoneSmemBitonicMax, st>>>(
         c->d_disks, c->slot_disk, c->key[0], c->val[0], c->id[b], c->rfix_longs, c->rfix_count, c->rfix_count + 1);
     ZoneArgs A;
@@ -840,10 +850,7 @@ cudaError_t launch_regrid(mcd_ctx *c)
     A.n_alive = c->n_alive;
     A.rkey = c->key[0];
     A.rsrc = c->val[0];
-    A.m0 = c->m[b]; A.M0 = c->M[b]; A.r0 = c->r[b]; A.z0 = c->z[b]; A.id0 = c->id[b];
-    A.m1 = c->m[nb]; A.M1 = c->M[nb]; A.r1 = c->r[nb]; A.z1 = c->z[nb]; A.id1 = c->id[nb];
-    A.q0 = c->tracer ? c->q[b] : nullptr;
-    A.q1 = c->tracer ? c->q[nb] : nullptr;
+    A.col = col;
     A.cell_start = c->cell_start;
     A.cell_n = c->cell_n;
     A.cell_b = c->cell_b;
@@ -856,10 +863,7 @@ cudaError_t launch_regrid(mcd_ctx *c)
     A.gas_knots = c->gas_knots;
     A.gas_n = c->gas_n;
     k_zone<<<(unsigned)c->Z, kZoneThreads, zp.smem, st>>>(A);
-    k_dead_tail<<<gN, 256, 0, st>>>(c->d_disks, c->slot_disk, c->N, c->n_alive, c->val[0], c->m[b], c->M[b], c->r[b],
-                                    c->z[b], c->id[b], c->m[nb], c->M[nb], c->r[nb], c->z[nb], c->id[nb],
-                                    c->tracer ? c->q[b] : nullptr, c->tracer ? c->q[nb] : nullptr);
-    c->launches += 5 + 4 * kRadixUpperPasses;
+    c->launches += 4 + (scanned ? 3 : 2) * kRadixUpperPasses;
     return cudaGetLastError();
 }
 
