@@ -18,7 +18,8 @@ BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libmcd.so")
 SOURCES = ["mcd_capi.cu", "mcd_collide.cu", "mcd_collide_f32c2.cu", "mcd_collide_f32c4.cu", "mcd_collide_f32c8.cu",
            "mcd_collide_f32c16.cu", "mcd_collide_f32s1.cu", "mcd_collide_f32s2.cu", "mcd_collide_f32s1x.cu",
-           "mcd_collide_f32s2x.cu", "mcd_collide_f64.cu",
+           "mcd_collide_f32s2x.cu", "mcd_collide_f64c4.cu",
+           "mcd_collide_f64c8.cu", "mcd_collide_f64c16.cu",
            "mcd_collide_f32ws4.cu", "mcd_collide_f32ws10.cu", "mcd_regrid.cu", "mcd_transport.cu", "mcd_noalloc.cu",
            "mcd_diag.cu", "mcd_step.cu", "mcd_peaks.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -3,14 +3,14 @@
 // timed trial that picks each class's variant, and the probes.  The kernels
 // themselves are in mcd_collide.cuh, instantiated per (precision, swarms per
 // thread, exact total) in mcd_collide_f32s1.cu, mcd_collide_f32s2.cu, mcd_collide_f32s1x.cu,
-// mcd_collide_f32s2x.cu and mcd_collide_f64.cu, the mixed path's variants with
-// specialised warps (S = 1) in mcd_collide_chain.cuh
-// (mcd_collide_f32c2.cu, mcd_collide_f32c4.cu, mcd_collide_f32c8.cu,
-// mcd_collide_f32c16.cu), and the control-warp variants
+// mcd_collide_f32s2x.cu, the variants with specialised warps (S = 1) in
+// mcd_collide_chain.cuh (mixed: mcd_collide_f32c2.cu, mcd_collide_f32c4.cu,
+// mcd_collide_f32c8.cu, mcd_collide_f32c16.cu) and mcd_collide_chain64.cuh (FP64:
+// mcd_collide_f64c4.cu, mcd_collide_f64c8.cu, mcd_collide_f64c16.cu), and the control-warp variants
 // in mcd_collide_ws.cuh (mcd_collide_f32ws4.cu, mcd_collide_f32ws10.cu).
 #include <algorithm>
 
-#include "mcd_collide_chain.cuh"
+#include "mcd_collide_chain64.cuh"
 #include "mcd_collide_ws.cuh"
 
 namespace mcd {
@@ -222,8 +222,7 @@ static cudaError_t variant(int op, int S, int store, bool ramp, bool tracer, boo
                            size_t smem, cudaStream_t st, const CollideArgs *A, int *out)
 {
     if constexpr (sizeof(T) == 8) {
-        if (S != 1 || store == 1 || exact) return cudaErrorInvalidValue;
-        return collide_variant<double, 1, false>(op, store, ramp, tracer, grid, nthr, smem, st, A, out);
+        return cudaErrorInvalidValue;  // (FP64 launches are chain launches)
     } else {
         if (exact)
             return S == 2 ? collide_variant<float, 2, true>(op, store, ramp, tracer, grid, nthr, smem, st, A, out)
@@ -234,10 +233,19 @@ static cudaError_t variant(int op, int S, int store, bool ramp, bool tracer, boo
 }
 
 // the chain variants for launches of nsl swarm slots
+template <class T>
 static cudaError_t chain_variant(int op, int nsl, int store, bool ramp, bool tracer, unsigned grid, size_t smem,
                                  cudaStream_t st, const CollideArgs *A, int *out)
 {
     const int nthr = nsl + 32 * kChainRoles;
+    if constexpr (sizeof(T) == 8) {
+        switch (chain_slots(nsl)) {
+        case 4: return collide_chain64_variant<4>(op, store, ramp, tracer, grid, nthr, smem, st, A, out);
+        case 8: return collide_chain64_variant<8>(op, store, ramp, tracer, grid, nthr, smem, st, A, out);
+        case 16: return collide_chain64_variant<16>(op, store, ramp, tracer, grid, nthr, smem, st, A, out);
+        default: return cudaErrorInvalidValue;
+        }
+    }
     if (nsl <= 64)
         return collide_chain_variant<4, kChainSmallCtas>(op, store, ramp, tracer, grid, nthr, smem, st, A, out);
     switch (chain_slots(nsl)) {
@@ -324,8 +332,9 @@ static ClassLaunch class_launch(const CollideClass &k, int threads, int spt, int
     if (sizeof(T) == 4 && !threads && block_threads<T>(class_threads(k.n_hi, 1), exact) > kMaxCell) L.S = 2;
     L.store = usable_store<T>(k, dv_matrix >= 0 ? dv_matrix : k.store);
     L.nthr = block_threads<T>(threads ? threads : class_threads(k.n_hi, L.S), exact);
-    L.chain = sizeof(T) == 4 && L.S == 1 && !exact;
+    L.chain = sizeof(T) == 8 || (L.S == 1 && !exact);
     auto bytes = [&]() {
+        if (sizeof(T) == 8) return collide_chain64_smem_bytes(L.nthr, tracer != 0);
         return L.chain ? collide_chain_smem_bytes(L.nthr, tracer != 0, L.store, k.rows, k.W)
                        : collide_smem_bytes<T>(L.nthr, L.S, tracer != 0, L.store, k.rows, k.W, exact);
     };
@@ -367,7 +376,7 @@ template <class T>
 static cudaError_t launch_op(int op, const ClassLaunch &L, bool ramp, bool tracer, bool exact, unsigned grid,
                              cudaStream_t st, const CollideArgs *A, int *out)
 {
-    if (L.chain) return chain_variant(op, L.nthr, L.store, ramp, tracer, grid, L.smem, st, A, out);
+    if (L.chain) return chain_variant<T>(op, L.nthr, L.store, ramp, tracer, grid, L.smem, st, A, out);
     if (L.ws) return ws_variant(op, L.pl, L.store, ramp, tracer, grid, L.nthr, L.smem, st, A, out);
     return variant<T>(op, L.S, L.store, ramp, tracer, exact, grid, L.nthr, L.smem, st, A, out);
 }
@@ -475,11 +484,10 @@ static cudaError_t prepare_impl(mcd_ctx *c)
     if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     int smin = optin;
-    for (int exact = 0; exact <= (sizeof(T) == 4 ? 1 : 0); ++exact)
-        for (int S = 1; S <= (sizeof(T) == 4 ? 2 : 1); ++S)
+    for (int exact = 0; sizeof(T) == 4 && exact <= 1; ++exact)
+        for (int S = 1; S <= 2; ++S)
             for (int store = 0; store <= 2; ++store) {
-                if (sizeof(T) == 8 && store == 1) continue;
-                if (sizeof(T) == 4 && S == 1 && !exact && store != 1) continue;  // (the chain variants, below)
+                if (S == 1 && !exact && store != 1) continue;  // (the chain variants, below)
                 int st = 0;
                 if ((e = variant<T>(2, S, store, false, false, exact, 0, 0, 0, nullptr, nullptr, &st)) != cudaSuccess)
                     return e;
@@ -490,19 +498,19 @@ static cudaError_t prepare_impl(mcd_ctx *c)
                     return e;
                 smin = std::min(smin, dyn);
             }
-    if (sizeof(T) == 4)
-        for (int nsl : {64, 128, 256, 512})
-            for (int store = 0; store <= 2; ++store) {
-                int st = 0;
-                if ((e = chain_variant(2, nsl, store, false, false, 0, 0, nullptr, nullptr, &st)) != cudaSuccess)
-                    return e;
-                const int dyn = optin - st;
-                if (dyn <= 0) return cudaErrorInvalidValue;
-                if ((e = chain_variant(1, nsl, store, false, false, 0, (size_t)dyn, nullptr, nullptr, nullptr)) !=
-                    cudaSuccess)
-                    return e;
-                smin = std::min(smin, dyn);
-            }
+    for (int nsl : {64, 128, 256, 512})
+        for (int store = 0; store <= 2; ++store) {
+            if (sizeof(T) == 8 && store == 1) continue;
+            int st = 0;
+            if ((e = chain_variant<T>(2, nsl, store, false, false, 0, 0, nullptr, nullptr, &st)) != cudaSuccess)
+                return e;
+            const int dyn = optin - st;
+            if (dyn <= 0) return cudaErrorInvalidValue;
+            if ((e = chain_variant<T>(1, nsl, store, false, false, 0, (size_t)dyn, nullptr, nullptr, nullptr)) !=
+                cudaSuccess)
+                return e;
+            smin = std::min(smin, dyn);
+        }
     if (sizeof(T) == 4)  // the control-warp variants
         for (int pl : {4, 7, 10, 16})
             for (int store = 0; store <= 2; ++store) {

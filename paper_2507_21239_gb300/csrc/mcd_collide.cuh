@@ -212,6 +212,17 @@ __device__ __forceinline__ double sqrt64(double x)
     const double y = f2d_int(y0), t = x * y, e = fma(-t, y, 1.0);
     return fma(t, e * fma(0.375, e, 0.5), t);
 }
+// cbrt from FP32 (a to about 2^-21, 1/a alongside), then two Newton steps with
+// the FP32 derivative: an error of 2^-21 goes to 2^-41 and 2^-61
+__device__ __forceinline__ double cbrt64(double x)
+{
+    if (!in_f32_range(x)) return cbrt(x);
+    const float l3 = lg2_mufu(d2f_int(x)) * (1.0f / 3.0f), ia = ex2_mufu(-l3);
+    const double h = f2d_int(ia * ia * (1.0f / 3.0f));
+    double a = f2d_int(ex2_mufu(l3));
+    a = fma(fma(-a * a, a, x), h, a);
+    return fma(fma(-a * a, a, x), h, a);
+}
 // order of non-negative doubles through their bit patterns
 __device__ __forceinline__ double min_pos(double a, double b)
 {
@@ -239,19 +250,7 @@ __device__ __forceinline__ Part<double> make_part<double>(const CellK<double> &c
     const int cls = mb < __double_as_longlong(c.m_eta) ? 0 : (mb < __double_as_longlong(c.m_one) ? 1 : 2);
     q.mh = m;
     q.ml = 0.0;
-    const double x = c.cm_d * m;
-    if (in_f32_range(x)) {
-        // cbrt from FP32 (a0 to about 2^-21, 1/a0 alongside), then two Newton steps
-        // with the FP32 derivative: a error of 2^-21 goes to 2^-41 and 2^-61
-        const float l3 = lg2_mufu(d2f_int(x)) * (1.0f / 3.0f), ia = ex2_mufu(-l3);
-        const double h = f2d_int(ia * ia * (1.0f / 3.0f));
-        double a = f2d_int(ex2_mufu(l3));
-        a = fma(fma(-a * a, a, x), h, a);
-        a = fma(fma(-a * a, a, x), h, a);
-        q.a = a;
-    } else {
-        q.a = cbrt(x);
-    }
+    q.a = cbrt64(c.cm_d * m);
     q.S = stk ? c.Cst * q.a * q.a : c.Cep * q.a;
     q.Sl = 0.0;
     q.p = rcp64(fma(q.S, q.S, 1.0));

@@ -176,6 +176,7 @@ struct PhiloxRounds {
         c0 = n0, c1 = l1, c2 = n2, c3 = l0;
         k0 += kPhiloxW0, k1 += kPhiloxW1;
     }
+    __device__ __forceinline__ U4 words() const { return U4{{c0, c1, c2, c3}}; }
     __device__ __forceinline__ Draw<float> draw(float sc) const { return make_draw(U4{{c0, c1, c2, c3}}, sc); }
 };
 
@@ -349,7 +350,8 @@ __device__ __forceinline__ Part<float> part_select(bool other, const Part<float>
 
 // the outcomes of mass m that do not depend on the partner: a grouped partner
 // of total mass dmm = dm m sticks, or erodes
-__device__ __forceinline__ double ready_mass(const CellK<float> &c, double m, double dmm, bool erodes)
+template <class T>
+__device__ __forceinline__ double ready_mass(const CellK<T> &c, double m, double dmm, bool erodes)
 {
     if (!erodes) return m + dmm;
     const double me = m - c.chi * dmm;
