@@ -61,6 +61,17 @@ struct alignas(16) Part {
     int32_t fl;        // turbulence regime (0,1,2) | stokes << 2
 };
 
+// FP64: what a pair can read instead of form, its instructions being what an event costs
+template <>
+struct alignas(16) Part<double> {
+    double a, im, Mv, gi;
+    double S, S2, S3;  // Stokes number, S^2, 2 S^3
+    double P2, q, qz;  // 1/(1+S^2)^2, 1/(1+S), Omega |z| (and the settling form's 1/(1+S)^2)
+    double bm;         // thermal motion's part of dv^2
+    double mh, ad;     // mass, (a - a_sw) for Stokes-law swarms
+    int32_t fl;
+};
+
 // ---- per-cell constants ----------------------------------------------------------
 template <class T>
 struct CellK {
@@ -70,6 +81,7 @@ struct CellK {
     T invVsc_t, dm_t, vfrag_t, m0_t, fe_t;
     int32_t kmode, settle, fe_zero;
     double m_sw, m_eta, m_one, m0, V, sc, invVsc, vfrag, ratio, chi, dm, fe, cm_d;
+    double CepCm, CstCm, soz;  // FP64 path: Cep cm, Cst cm, Omega |z|
 };
 static_assert(sizeof(CellK<double>) <= kCellKBytes && sizeof(CellK<float>) <= kCellKBytes, "cell constants");
 
@@ -105,6 +117,8 @@ __device__ CellK<T> make_cell(const mcd_disk_params &P, GasTab tab, double rc, d
     split(c.m_eta, c.meta_h, c.meta_l);
     split(c.m_one, c.mone_h, c.mone_l);
     c.cm_d = cm;
+    c.CepCm = Cep * cm;
+    c.CstCm = Cst * cm;
     c.asw = (T)g.asw;
     c.vg2 = (f & MCD_DV_TURB) ? (T)g.vg2 : (T)0;
     c.Se = (T)g.St_eta;
@@ -113,6 +127,7 @@ __device__ CellK<T> make_cell(const mcd_disk_params &P, GasTab tab, double rc, d
     c.e1 = (f & MCD_DV_PHI) ? (T)(g.etavk * g.etavk) : (T)0;
     double oz = g.Omega * fabs(zc);
     c.oz2 = (f & MCD_DV_SET) ? (T)(oz * oz) : (T)0;
+    c.soz = (f & MCD_DV_SET) ? oz : 0.0;
     c.Kc = (T)P.K_const;
     c.pi = (T)kPI;
     c.kmode = P.kernel_mode;
@@ -186,9 +201,10 @@ __device__ __forceinline__ float lg2_mufu(float x)
 // take one third-order step (Householder's iterations), three and five FP64
 // instructions, instead of the correctly rounded routines.  Values outside the
 // FP32 range take the plain operation (a branch that rates do not take).
-// A 0D cell of 200 swarms 9.5 -> 8.2 ms, 16 cells of 4 x 100 25.6 -> 21.4 ms a
-// step, 256 x 16 of 200 14.8 -> 11.0 ms; error of K against quadruple precision,
-// rms over the regimes, 1.92 -> 1.82e-16 (the correctly rounded routines round
+// With every thread doing all of an event: a 0D cell of 200 swarms 9.5 -> 8.2 ms,
+// 16 x 4 cells of 100 25.6 -> 21.4 ms in eight steps, 256 x 16 of 200 14.8 -> 11.0
+// ms a step.  Error of K against quadruple precision, rms in four gas regimes:
+// 1.87 to 1.92e-16 -> 1.74 to 1.86e-16 (the correctly rounded routines round
 // more intermediate results).
 __device__ __forceinline__ bool in_f32_range(double x)
 {
@@ -249,17 +265,24 @@ __device__ __forceinline__ Part<double> make_part<double>(const CellK<double> &c
     const bool stk = mb >= __double_as_longlong(c.m_sw);
     const int cls = mb < __double_as_longlong(c.m_eta) ? 0 : (mb < __double_as_longlong(c.m_one) ? 1 : 2);
     q.mh = m;
-    q.ml = 0.0;
-    q.a = cbrt64(c.cm_d * m);
-    q.S = stk ? c.Cst * q.a * q.a : c.Cep * q.a;
-    q.Sl = 0.0;
-    q.p = rcp64(fma(q.S, q.S, 1.0));
-    q.q = rcp64(1.0 + q.S);
-    q.im = rcp64(m);
-    q.ad = stk ? c.cm_d * (m - c.m_sw) / ((q.a * q.a + c.asw * c.asw) + q.a * c.asw) : 0.0;
     q.Mv = Mv;
-    q.gi = c.dm > 0.0 ? rcp64(c.dm * m) : (double)INFINITY;
     q.fl = cls | ((int)stk << 2);
+    q.im = rcp64(m);
+    q.gi = c.dm > 0.0 ? rcp64(c.dm * m) : (double)INFINITY;
+    if (c.kmode == 1) {  // the constant kernel: rates and outcomes take masses alone
+        q.a = q.S = q.S2 = q.S3 = q.P2 = q.q = q.qz = q.bm = q.ad = 0.0;
+        return q;
+    }
+    q.a = cbrt64(c.cm_d * m);
+    q.S = (stk ? c.Cst * q.a : c.Cep) * q.a;
+    q.S2 = q.S * q.S;
+    q.S3 = q.S2 * (q.S + q.S);
+    const double p = rcp64(1.0 + q.S2);
+    q.P2 = p * p;
+    q.q = rcp64(1.0 + q.S);
+    q.qz = c.settle ? q.q * q.q * c.soz : c.soz;
+    q.bm = c.cbm * q.im;
+    q.ad = stk ? c.cm_d * (m - c.m_sw) / ((q.a * q.a + c.asw * c.asw) + q.a * c.asw) : 0.0;
     return q;
 }
 
@@ -388,40 +411,38 @@ __device__ __forceinline__ T pair_dv(const C &c, const Part<T> &u, const Part<T>
         *K = kern_of<T>(c, u.a, v.a, dv);
         return dv;
     } else {
-        // FP64, about 46 FP64 instructions for the common case (two Epstein swarms,
+        // FP64, about 40 FP64 instructions for the common case (two Epstein swarms,
         // regime II) against some 150 with correctly rounded divisions and square
-        // root, and the warp's other regimes only where one of its lanes needs them.
+        // root and nothing read from the caches, and the warp's other regimes only
+        // where one of its lanes needs them.
         const unsigned lanes = __activemask();
         const T s2 = u.a + v.a;
-        const T da = c.cm * fabs(u.mh - v.mh) * rcp64(fma(s2, s2, -(u.a * v.a)));  // a_u - a_v from the cubes
-        T D = c.Cep * da;
+        const T G = fabs(u.mh - v.mh) * rcp64(fma(s2, s2, -(u.a * v.a)));  // cm G = a_u - a_v from the cubes
+        T D = c.CepCm * G;
         if (__any_sync(lanes, su | sv)) {
             const T as = su ? u.a : v.a, ads = su ? u.ad : v.ad;
-            D = (su & sv) ? c.Cst * s2 * da : ((su | sv) ? c.Cst * fma(as, ads, c.asw * da) : D);
+            D = (su & sv) ? c.CstCm * s2 * G : ((su | sv) ? c.Cst * fma(as, ads, c.asw * (c.cm * G)) : D);
         }
         const T S1 = max_pos(u.S, v.S), S2 = min_pos(u.S, v.S), s = S1 + S2, D2 = D * D;
-        T t0 = c.cbm * (u.im + v.im);
+        T t0 = u.bm + v.bm;
         if (__double_as_longlong(c.vg2) > 0) {
             if (__any_sync(lanes, cls == 1)) {
                 // regime II with eps = S2/S1 cleared from the fractions, as in FP32
                 const T A1 = fma((T)kYA, S1, S2);
-                const T num = fma(A1 * (S1 * S1), (T)(2.0 / (1.0 + kYA)), (T)2 * S2 * (S2 * S2));
+                const T num = fma(A1 * max_pos(u.S2, v.S2), (T)(2.0 / (1.0 + kYA)), min_pos(u.S3, v.S3));
                 const T t2 = fma(num, rcp64(s * A1), fma((T)(2.0 * kYA - 1.0), S1, -S2));
                 t0 = cls == 1 ? fma(c.vg2, t2, t0) : t0;
             }
             if (__any_sync(lanes, cls == 2)) t0 = cls == 2 ? fma(c.vg2, u.q + v.q, t0) : t0;
             if (__any_sync(lanes, cls == 0)) {
-                const T g1 = c.vg2 * fma(S1, S2, c.Se * s) * rcp64(s * ((S1 + c.Se) * (S2 + c.Se)));
+                // (S1 + Se)(S2 + Se) = X + Se^2
+                const T X = fma(S1, S2, c.Se * s);
+                const T g1 = c.vg2 * X * rcp64(s * fma(c.Se, c.Se, X));
                 t0 = cls == 0 && __double_as_longlong(s) > 0 ? fma(D2, g1, t0) : t0;
             }
         }
-        const T pp = u.p * v.p, om = fma(-u.S, v.S, (T)1);
-        T cz = c.oz2;
-        if (c.settle) {
-            const T qq = u.q * v.q;
-            cz *= qq * qq;
-        }
-        const T coef = fma(pp * pp, fma(c.e1 * s, s, c.e4 * om * om), cz);
+        const T om = fma(-u.S, v.S, (T)1);
+        const T coef = fma(u.P2 * v.P2, fma(c.e1 * s, s, c.e4 * om * om), u.qz * v.qz);
         const T dv = sqrt64(fma(D2, coef, t0));
         *K = c.pi * s2 * s2 * dv;
         return dv;

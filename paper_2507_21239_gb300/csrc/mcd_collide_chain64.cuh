@@ -7,7 +7,7 @@
 // the FP64 instructions of the busiest sub-partition, and what one lane alone
 // needs (the clock, the outcome, a swarm's cache) costs as much as a whole row.
 //  * worker warps (thread k owns swarm k) only form row i, the new row and
-//    column and their weights, some 60 instructions per event, 46 of them the
+//    column and their weights, some 52 instructions per event, 40 of them the
 //    new pair;
 //  * prefixes and sums over a group of 32 swarms run in 64-bit integers at the
 //    scale of the group's largest rate (group_prefix64): no FP64 instruction,
@@ -24,7 +24,9 @@
 // Measured, heaviest cell, us per event (every thread doing all of it with
 // block-wide scans -> this): 20 swarms 6.7 -> 5.0, 100: 7.2 -> 5.4, 200: 9.9 ->
 // 7.4, 300: 13.3 -> 9.4, 400: 16.6 -> 11.3, 512: 19.3 -> 13.3; recomputing row
-// i 13.8 -> 11.6 at 200.  Many light cells, which the units bound whatever the
+// i 13.8 -> 11.6 at 200.  With powers of S and the terms of one swarm read from
+// its cache, and the cache of a general outcome formed by the whole choice
+// warp: 4.7, 5.1, 6.8 (200), 10.6 (400), 12.4 (512); recomputing 10.3 at 200.  Many light cells, which the units bound whatever the
 // layout, take the same: 32,768 cells of 40 swarms 7.7 ms, of 64 14.7 ms.
 #pragma once
 #include "mcd_collide_chain.cuh"
@@ -140,37 +142,45 @@ __device__ __forceinline__ bool choose64(double bs, const double *pf, double u, 
 }
 
 // The cache of mass m in place, by a warp: lanes 4 e + f hold outcome e's mass
-// and write its field f (1/(1+S^2), 1/(1+S), 1/m, 1/(dm m)), so that one
-// reciprocal serves all of them; the same expressions as make_part<double>.
+// (a general outcome: lanes f) and write its field f (from 1/(1+S^2), 1/(1+S),
+// 1/m, 1/(dm m)), so that one reciprocal serves all of them; the same
+// expressions as make_part<double>.
 __device__ __forceinline__ void make_ready64(const CellK<double> &c, double m, double dmm, double Mv, Part<double> *dst,
                                              int f, bool store)
 {
     const long long mb = __double_as_longlong(m);
     const bool stk = mb >= __double_as_longlong(c.m_sw);
     const int cls = mb < __double_as_longlong(c.m_eta) ? 0 : (mb < __double_as_longlong(c.m_one) ? 1 : 2);
-    const double a = cbrt64(c.cm_d * m);
+    const bool flat = c.kmode == 1;  // the constant kernel: masses alone
+    const double a = flat ? 0.0 : cbrt64(c.cm_d * m);
     const double S = (stk ? c.Cst * a : c.Cep) * a;
-    double x = fma(S, f == 0 ? S : 1.0, 1.0);
+    const double S2 = S * S;
+    double x = 1.0 + (f == 0 ? S2 : S);
     x = f == 2 ? m : (f == 3 ? dmm : x);
     double y = rcp64(x);
     if (f == 3 && !(__double_as_longlong(c.dm) > 0)) y = (double)INFINITY;
+    const double z = y * (f == 2 ? c.cbm : y);  // (f == 3: not used)
     double ad = 0.0;
-    if (__any_sync(0xffffffffu, stk))
+    if (__any_sync(0xffffffffu, stk && !flat))
         ad = stk ? c.cm_d * (m - c.m_sw) / ((a * a + c.asw * c.asw) + a * c.asw) : 0.0;
     if (!store) return;
-    double *const field = f == 0 ? &dst->p : (f == 1 ? &dst->q : (f == 2 ? &dst->im : &dst->gi));
-    *field = y;
     if (f == 0) {
+        dst->P2 = z;
         dst->a = a;
         dst->S = S;
-        dst->Sl = 0.0;
+        dst->S2 = S2;
+        dst->S3 = S2 * (S + S);
     } else if (f == 1) {
+        dst->q = y;
+        dst->qz = c.settle ? z * c.soz : c.soz;
         dst->mh = m;
-        dst->ml = 0.0;
     } else if (f == 2) {
+        dst->im = y;
+        dst->bm = z;
         dst->Mv = Mv;
         dst->ad = ad;
     } else {
+        dst->gi = y;
         dst->fl = cls | ((int)stk << 2);
     }
 }
@@ -342,13 +352,17 @@ __device__ __forceinline__ void chain64_cell(const CollideArgs &A, const int64_t
                         mnew = outcome_ramp<T>(c, mmi.x, mj, (T)0, (T)0, mmi.y, dvij, dr.u3, vlo, kind);
                     else
                         mnew = outcome<T>(c, mmi.x, mj, (T)0, (T)0, mmi.y, dvij, dr.u3, kind);
-                    ready[gen] = make_part<T>(c, mnew, Mvi);
-                    mready[gen] = make_double2(mnew, __dmul_rn(c.dm, mnew));
                 } else {
                     mnew = ready_mass(c, mmi.x, mmi.y, !stick);  // (the mass warp may still be at work on mready)
                 }
                 if constexpr (TRACER)
                     qnew = tracer_update(mmi.x, mj, qsh[i], qsh[j], dgt(mmi.y, mj) ? mmi.y : mj, mnew, kind, c.chi);
+            }
+            const unsigned gm = __ballot_sync(0xffffffffu, jhere && !grouped);
+            if (gm) {  // the cache of a general outcome, by the whole warp
+                const double m = __shfl_sync(0xffffffffu, mnew, __ffs(gm) - 1), dmm = __dmul_rn(c.dm, m);
+                make_ready64(c, m, dmm, Mvi, ready + gen, lane & 3, lane < 4);
+                if (lane == 0) mready[gen] = make_double2(m, dmm);
             }
             __syncwarp();
             bar_sync(kBarEvent, nthr);
