@@ -334,11 +334,11 @@ def collide_rooflines(n_c, ev_c, n_steps, collide_ms, pk, fp32_unit_peak):
     sm_bytes = sum(collide_smem_bytes(n_c[k], ev_c[k]) for k in range(n_steps)) / n_steps
     t = collide_ms * 1e-3
     alu = {"bound": "alu", "achieved": entries * FLOPS_PER_ENTRY / t / 1e12, "peak": fp32_unit_peak,
-           "unit": "TFLOP/s", "traffic": measured_traffic("k_collide<float>"), "kernel": "k_collide<float>",
+           "unit": "TFLOP/s", "traffic": measured_traffic("k_collide_chain"), "kernel": "k_collide_chain",
            "peak_source": "152 SMs x 128 FP32 lanes x 2 flop x max SM clock (MEASURED_PEAKS.json)",
            "work": f"{FLOPS_PER_ENTRY} flop x {entries:.4g} kernel entries per step"}
     smem = {"bound": "smem", "achieved": sm_bytes / t / 1e9, "peak": pk["smem_gbs"], "unit": "GB/s",
-            "traffic": None, "kernel": "k_collide<float>",
+            "traffic": None, "kernel": "k_collide_chain",
             "peak_source": "measured in this run (mcd_probe_peaks shared-memory read loop)",
             "work": f"{sm_bytes:.4g} algorithmic shared-memory bytes per step"}
     for x in (alu, smem):

@@ -202,8 +202,8 @@ __device__ __forceinline__ float lg2_mufu(float x)
 // instructions, instead of the correctly rounded routines.  Values outside the
 // FP32 range take the plain operation (a branch that rates do not take).
 // With every thread doing all of an event: a 0D cell of 200 swarms 9.5 -> 8.2 ms,
-// 16 x 4 cells of 100 25.6 -> 21.4 ms in eight steps, 256 x 16 of 200 14.8 -> 11.0
-// ms a step.  Error of K against quadruple precision, rms in four gas regimes:
+// four steps of 16 x 4 cells of 100 25.6 -> 21.4 ms, a step of 256 x 16 of 200
+// 59.3 -> 44.2 ms.  Error of K against quadruple precision, rms in four gas regimes:
 // 1.87 to 1.92e-16 -> 1.74 to 1.86e-16 (the correctly rounded routines round
 // more intermediate results).
 __device__ __forceinline__ bool in_f32_range(double x)
