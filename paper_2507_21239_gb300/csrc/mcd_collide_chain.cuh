@@ -53,9 +53,18 @@
 namespace mcd {
 
 // named barriers (0 is __syncthreads): count is the number of threads that
-// arrive or wait
-__device__ __forceinline__ void bar_sync(int id, int count) { asm volatile("barrier.cta.sync.aligned %0, %1;" ::"r"(id), "r"(count) : "memory"); }
-__device__ __forceinline__ void bar_arrive(int id, int count) { asm volatile("barrier.cta.arrive.aligned %0, %1;" ::"r"(id), "r"(count) : "memory"); }
+// arrive or wait.  The .aligned forms want the whole warp at one instruction;
+// what precedes them may depend on the lane, so each brings the warp together first.
+__device__ __forceinline__ void bar_sync(int id, int count)
+{
+    __syncwarp();
+    asm volatile("barrier.cta.sync.aligned %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id, int count)
+{
+    __syncwarp();
+    asm volatile("barrier.cta.arrive.aligned %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
 // kBarNew: the new row posted (workers arrive; the clock warp waits); kBarRead:
 // i's new cache read (workers arrive; the mass warp waits); kBarRates: prefixes
 // of R posted, the fresh R_i, masses and caches too (workers and mass warp
@@ -515,13 +524,11 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
                     sh.pick.x = -2;
                     sh.sel.x = -2;
                 }
-                __syncwarp();
                 bar_arrive(kBarI, nsl + 32);
                 bar_sync(kBarEvent, nthr);
                 break;
             }
             if (any ? ihere : lane == 0) sh.sel.x = any ? i : n - 1;  // (no bracket, rates not finite: stay in bounds)
-            __syncwarp();
             bar_arrive(kBarI, nsl + 32);
             i = sh.sel.x;
             const double2 mmi = mm[i];
@@ -559,7 +566,6 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
                 if constexpr (TRACER)
                     qnew = tracer_update(mmi.x, mj, qsh[i], qsh[j], dgt(mmi.y, mj) ? mmi.y : mj, mnew, kind, c.chi);
             }
-            __syncwarp();
             bar_sync(kBarEvent, nthr);
             const int2 pick = sh.pick;
             if (pick.x < 0 || pick.y) {
@@ -578,7 +584,6 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
                         A.log_m[ev] = mnew;
                     }
                 }
-                __syncwarp();
             }
             pend = i;
             ++ev;
@@ -608,7 +613,6 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
             const T Mvi = ready[pick.x].Mv;
             const double2 mi = mready[pick.x];
             if (lane == 0) mm[i] = mi;
-            __syncwarp();
             if (--until_rebuild == 0) {
                 bar_arrive(kBarBuild, nsl + 32);
                 until_rebuild = reb;
@@ -623,7 +627,6 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
                 ready[lane * nsl + i] = pnew;
                 mready[lane * nsl + i] = make_double2(mnew, dmnew);
             }
-            __syncwarp();
             bar_arrive(kBarReady, nsl + 32);
         }
     } else if (w > ng + 1) {  // ---- the clock warp ----
@@ -640,7 +643,6 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
             load_words<32>(sh.ys, z);
             const T Rp = tree_down<32>(z);
             if (lane == 0) sh.sel.y = __float_as_int(Rp);
-            __syncwarp();
             bar_sync(kBarRates, nsl + 96);
             load_words<NW>(sh.ti + NW, all);
             const T tot = tree_down<NW>(all) + Rp;
@@ -658,7 +660,6 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
             if (q == 0) px.start((uint64_t)((ev | 31) + 1 + lane), dcell, step, A.seed, (uint64_t)disk);
             if (q < 10) px.round();
             if (q == 10) sh.ring[((ev | 31) + 1 + lane) & 63] = px.draw(sc);
-            __syncwarp();
             bar_sync(kBarEvent, nthr);
             const int2 pick = sh.pick;
             if (pick.x < 0 || pick.y) break;
@@ -708,7 +709,6 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
             pf[k] = x;
             if (lane == 31) sh.ti[2 * NW - ng + w] = x;
             if (STORE != 0 && act && pend >= 0) Dm[at] = dvn;
-            __syncwarp();
             bar_arrive(kBarRates, nsl + 96);
             R.s = upd ? Rn.s : R.s;
             R.c = upd ? Rn.c : R.c;
@@ -737,7 +737,6 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
             x = group_prefix(xw, act ? Kold * weight<T>(pi, pk) : (T)0);
             pf[k] = x;
             if (lane == 31) sh.tj[2 * NW - ng + w] = x;
-            __syncwarp();
             bar_arrive(kBarRow, nsl + 32);
             const T colo = Kold * weight<T>(pk, pi);
             // (3) meanwhile, for the ready outcome of the kind that came last: the new
@@ -770,7 +769,6 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
             if (AHEAD && hit) {
                 hi = his;
                 rn[k] = rebuild ? (T)0 : rows;
-                __syncwarp();
                 bar_arrive(kBarNew, nsl + 32);
                 Rn = Rs;
             } else {
@@ -779,7 +777,6 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
                 pk = part_select(k == i, pn, pk);
                 if (!hit) pair_flat1<false>(pc, false, pk, pn, dvn, Knew);
                 rn[k] = act && !rebuild ? Knew * weight<T>(pn, pk) : (T)0;
-                __syncwarp();
                 bar_arrive(kBarNew, nsl + 32);
                 Rn = R;
                 Rn.update(Knew * weight<T>(pk, pn), colo);

@@ -312,7 +312,6 @@ __device__ __forceinline__ void chain64_cell(const CollideArgs &A, const int64_t
                     sh.sel = -2;
                     sh.Rp = Rp;
                 }
-                __syncwarp();
                 bar_arrive(kBarI, nsl + 32);
                 bar_sync(kBarEvent, nthr);
                 break;
@@ -321,7 +320,6 @@ __device__ __forceinline__ void chain64_cell(const CollideArgs &A, const int64_t
                 sh.sel = any ? i : n - 1;  // (no bracket, rates not finite: stay in bounds)
                 sh.Rp = Rp;
             }
-            __syncwarp();
             bar_arrive(kBarI, nsl + 32);
             i = sh.sel;
             const double2 mmi = mm[i];
@@ -364,7 +362,6 @@ __device__ __forceinline__ void chain64_cell(const CollideArgs &A, const int64_t
                 make_ready64(c, m, dmm, Mvi, ready + gen, lane & 3, lane < 4);
                 if (lane == 0) mready[gen] = make_double2(m, dmm);
             }
-            __syncwarp();
             bar_sync(kBarEvent, nthr);
             const int2 pick = sh.pick;
             if (pick.x < 0 || pick.y) {
@@ -383,7 +380,6 @@ __device__ __forceinline__ void chain64_cell(const CollideArgs &A, const int64_t
                         A.log_m[ev] = mnew;
                     }
                 }
-                __syncwarp();
             }
             pend = i;
             ++ev;
@@ -413,7 +409,6 @@ __device__ __forceinline__ void chain64_cell(const CollideArgs &A, const int64_t
             const T Mvi = ready[pick.x].Mv;
             const double2 mi = mready[pick.x];
             if (lane == 0) mm[i] = mi;
-            __syncwarp();
             if (--until_rebuild == 0) {
                 bar_arrive(kBarBuild, nsl + 32);
                 until_rebuild = reb;
@@ -425,7 +420,6 @@ __device__ __forceinline__ void chain64_cell(const CollideArgs &A, const int64_t
             bar_sync(kBarRead, nsl + 32);
             make_ready64(c, mnew, dmnew, Mvi, ready + e * nsl + i, lane & 3, lane < 8);
             if (lane < 8 && (lane & 3) == 0) mready[e * nsl + i] = make_double2(mnew, dmnew);
-            __syncwarp();
         }
     } else if (w == ng + kRoleClock) {  // ---- the clock warp ----
         const double t_end = A.t_end_from_state ? A.state->t + A.state->dt : A.t_end_fixed;
@@ -450,7 +444,6 @@ __device__ __forceinline__ void chain64_cell(const CollideArgs &A, const int64_t
             if (q == 0) px.start((uint64_t)((ev | 31) + 1 + lane), dcell, step, A.seed, (uint64_t)disk);
             if (q < 10) px.round();
             if (q == 10) sh.ring[((ev | 31) + 1 + lane) & 63] = make_draw(px.words(), sc);
-            __syncwarp();
             bar_sync(kBarEvent, nthr);
             const int2 pick = sh.pick;
             if (pick.x < 0 || pick.y) break;
@@ -482,7 +475,6 @@ __device__ __forceinline__ void chain64_cell(const CollideArgs &A, const int64_t
             T x = group_prefix64(hi);
             pf[k] = x;
             if (lane == 31) sh.tot[0][w] = x;
-            __syncwarp();
             bar_arrive(kBarRates, nsl + 96);
             bar_sync(kBarI, nsl + 32);
             const int sel = sh.sel, i = max(sel, 0);
@@ -505,7 +497,6 @@ __device__ __forceinline__ void chain64_cell(const CollideArgs &A, const int64_t
             x = group_prefix64(act ? Kold * weight<T>(pi, pk) : (T)0);
             pf[k] = x;
             if (lane == 31) sh.tot[2][w] = x;
-            __syncwarp();
             bar_arrive(kBarRow, nsl + 32);
             const T colo = Kold * weight<T>(pk, pi);
             bar_sync(kBarEvent, nthr);
@@ -514,7 +505,6 @@ __device__ __forceinline__ void chain64_cell(const CollideArgs &A, const int64_t
             // (3) the new row and column i: R_k += r_ki(new) - r_ki(old); R_i afresh
             const Part<T> pn = ready[pick.x];
             if (k == i) pk = pn;
-            __syncwarp();
             bar_arrive(kBarRead, nsl + 32);
             T Knew;
             const T dvn = pair_dv<T>(c, pk, pn, &Knew);
