@@ -210,10 +210,12 @@ __device__ __forceinline__ bool in_f32_range(double x)
 {
     return ((unsigned)(__double_as_longlong(x) >> 52) - 949u) <= 200u;  // positive, 2^-74 to 2^127
 }
-// 1 / b: with y good to 2^-22 and e = 1 - b y, y (1 + e + e^2) leaves e^3
+// 1 / b: with y good to 2^-22 and e = 1 - b y, y (1 + e + e^2) leaves e^3.  Above
+// 2^126 the reciprocal is an FP32 subnormal, which the special-function unit
+// flushes to 0, so b ends at 2^125 here (rounding b to FP32 may reach the limit).
 __device__ __forceinline__ double rcp64(double b)
 {
-    if (!in_f32_range(b)) return 1.0 / b;
+    if (((unsigned)(__double_as_longlong(b) >> 52) - 949u) > 198u) return 1.0 / b;
     float y0;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(d2f_int(b)));
     const double y = f2d_int(y0), e = fma(-b, y, 1.0);
