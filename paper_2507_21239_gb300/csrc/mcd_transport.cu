@@ -113,8 +113,10 @@ __device__ __forceinline__ void transport_fp64(const DiskC<double> &P, GasTab ta
     const double rho = (P.tr_flags & MCD_TR_ST_MIDPLANE) ? rho_mid : rho_mid * exp(-0.5 * s2 * s2);  // (St's density)
     const double irho = 1.0 / rho, lambda = P.lamc * irho, vth = 1.5957691216057308 * cs;
     const double a = cbrt(P.ca * m);
-    const double St = a < 2.25 * lambda ? P.rho_s * a * irho * (ics * (1.0 / 1.5957691216057308)) * Om
-                                        : 2.0 * P.rho_s * a * a / (4.5 * vth * lambda * rho) * Om;
+    double St = a < 2.25 * lambda ? P.rho_s * a * irho * (ics * (1.0 / 1.5957691216057308)) * Om
+                                  : 2.0 * P.rho_s * a * a / (4.5 * vth * lambda * rho) * Om;
+    // 35 and more scale heights up (rho below 2^-930) 1/rho may be infinite where St is not
+    if ((__double_as_longlong(rho) >> 52) < 93) St = P.rho_s * a / (rho * vth) * Om;
     const double rho_bm = sqrt(-2.0 * log(u01d(x.x[0])));
     double sn, cn;
     sincospi(2.0 * u01d(x.x[1]), &sn, &cn);
