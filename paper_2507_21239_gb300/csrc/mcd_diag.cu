@@ -4,13 +4,14 @@
 // per radial bin [edges[b], edges[b+1]), the swarm-mass-weighted sums of the
 // representative mass's first three powers and the particle count.
 //
-// Two paths.  Disks of more than kMomentsSplitMin particles are cut into parts
-// of consecutive slots, one CTA each: a CTA reads its particles once, finds every
-// particle's bin, and forms one set of sums for every bin between its first and
-// last; after a regrid the slots lie in radial zones, so that is one bin or two.
-// A second kernel adds the parts' sums bin by bin.  One CTA per bin that scans
-// all particles (the other path, for small disks, where a part or two would not
-// fill the chip either) leaves SMs idle and reads every particle once per bin.
+// Two paths.  Disks of many particles per bin (kMomentsSplitMin, kMomentsPerBin) are
+// cut into parts of consecutive slots, one CTA each: a CTA finds the first and last
+// bin of its particles in one pass and forms the sums of each bin between them in a
+// pass of its own; after a regrid the slots lie in radial zones, so that is one bin
+// or two, and on particles in no order every bin.  A second kernel adds the parts'
+// sums bin by bin.  One CTA per bin that scans all particles (the other path, for
+// small disks and many bins) leaves SMs idle with few bins and reads every particle
+// once per bin.
 // Bound by the FP64 unit (an instruction per 16 SM cycles): 19 instructions per
 // particle and bin pass, so parts are small enough (1,024 particles) to even the
 // SMs out.  Both diagnostics of 819,200 particles (32 bins; a 64 x 96 map), calls
@@ -120,7 +121,16 @@ __device__ __forceinline__ NSum block_nsum4(const NSum (&a)[4], double2 (*sh)[4]
     return r;
 }
 
-constexpr int64_t kMomentsSplitMin = 16384;
+// Where the parts pay.  A pass over one bin of a part takes some 9 us whatever the
+// part's size (the block's sum is what it waits for), so with many bins per part
+// the CTA per bin is faster: at 1,536 particles per bin 65,536 particles take 142
+// (parts) against 153 us in zone order and 366 against 658 shuffled, at 1,024 181
+// against 142 and 491 against 621.  Parts larger than 1,024 (above 113 bins, so
+// that the records fit) are fewer and make longer passes: 204,800 particles at
+// 1,536 per bin 365 against 290 us, at 2,048 (100 bins) 217 against 351.  Disks of up
+// to 16,384 particles (80 to 155 us at 12,288) keep the CTA per bin.
+constexpr int64_t kMomentsSplitMin = 16384, kMomentsPart = 1024;
+constexpr int64_t kMomentsPerBin = 1536, kMomentsPerBinLarge = 2048;
 // a part's record of one bin: four compensated sums and the count
 struct MomentsPart {
     double s[4], c[4];
@@ -380,12 +390,13 @@ cudaError_t launch_moments(mcd_ctx *c, int disk, int nbins)
     const double *m = c->m[b] + D.p_off, *M = c->M[b] + D.p_off, *r = c->r[b] + D.p_off;
     // parts of P particles: their records and their bins' ranges take the sort's key
     // buffers (free between regrids)
-    int64_t P = 1024;
+    int64_t P = kMomentsPart;
     auto fits = [&](int64_t p) {
         return (size_t)((D.n0 + p - 1) / p) * nbins * sizeof(MomentsPart) <= sizeof(uint64_t) * (size_t)D.n0;
     };
     while (P < D.n0 && !fits(P)) P *= 2;
-    if (D.n0 > kMomentsSplitMin && fits(P) && P <= D.n0 / 4) {
+    const int64_t per_bin = P == kMomentsPart ? kMomentsPerBin : kMomentsPerBinLarge;
+    if (D.n0 > kMomentsSplitMin && D.n0 >= per_bin * nbins && fits(P) && P <= D.n0 / 4) {
         const int parts = (int)((D.n0 + P - 1) / P);
         MomentsPart *rec = reinterpret_cast<MomentsPart *>(c->key[0] + D.p_off);
         int2 *range = reinterpret_cast<int2 *>(c->key[1] + D.p_off);
