@@ -216,6 +216,14 @@ __device__ __forceinline__ Part<float> make_part_rn(const CellK<float> &c, doubl
     split_f64(m, mh, ml);
     q.mh = mh;
     q.ml = ml;
+    q.im = rcp_ftz(mh);
+    q.Mv = Mv;
+    q.gi = c.dm_t > 0.0f ? rcp_ftz(__fmul_rn(c.dm_t, mh)) : INFINITY;
+    if (c.kmode == 1) {  // the constant kernel: rates and outcomes take masses alone
+        q.a = q.S = q.Sl = q.p = q.q = q.ad = 0.0f;
+        q.fl = renewed;
+        return q;
+    }
     const bool stk = !pair_lt(mh, ml, c.msw_h, c.msw_l);
     const int cls = pair_lt(mh, ml, c.meta_h, c.meta_l) ? 0 : (pair_lt(mh, ml, c.mone_h, c.mone_l) ? 1 : 2);
     // x = cm m as a (hi, lo) pair, then a = cbrt(x) to about 2^-44: FP32 cube
@@ -238,19 +246,17 @@ __device__ __forceinline__ Part<float> make_part_rn(const CellK<float> &c, doubl
     q.Sl = __fsub_rn(Se, __fsub_rn(q.S, Sh));
     q.p = rcp_ftz(__fmaf_rn(q.S, q.S, 1.0f));
     q.q = rcp_ftz(__fadd_rn(1.0f, q.S));
-    q.im = rcp_ftz(mh);
     // a - a_sw = cm (m - m_sw) / (a^2 + a a_sw + a_sw^2), m - m_sw from the pairs
     const float dsw = __fadd_rn(__fsub_rn(mh, c.msw_h), __fsub_rn(ml, c.msw_l));
     q.ad = stk ? __fmul_rn(__fmul_rn(c.cm, dsw), rcp_ftz(__fmaf_rn(a0, c.asw, __fmaf_rn(c.asw, c.asw, p2)))) : 0.0f;
-    q.Mv = Mv;
-    q.gi = c.dm_t > 0.0f ? rcp_ftz(__fmul_rn(c.dm_t, mh)) : INFINITY;
     q.fl = cls | ((int)stk << 2) | renewed;
     return q;
 }
 
-// pair_dv<float> of N pairs (u, v) without a branch: every case evaluated and
-// selected (the constant kernel too), step by step for all N, so that the pairs
-// fill each other's latencies.  Every rounding is explicit, so the bits depend
+// pair_dv<float> of N pairs (u, v) without a branch but the constant kernel's (the
+// same for the whole cell; with every term formed for it too a 0D cell of 400 swarms
+// took 6.1 ms to t = 100, now 3.9): every other case evaluated and selected, step by
+// step for all N, so that the pairs fill each other's latencies.  Every rounding is explicit, so the bits depend
 // neither on the store nor on the warp that forms them; they are pair_dv's,
 // except that dv below 1e-19 cm/s (dv^2 no normal number) counts as 0.  EARLY:
 // with early set, a pair of two swarms that no event of this chain has renewed
@@ -263,6 +269,10 @@ __device__ __forceinline__ void pair_flat(const PairK<float> &c, bool early, con
     typedef float T;
     T da[N], D[N], S1[N], S2[N], s[N], g1[N], t2[N], t3[N], coef[N], t0[N];
 #define MCD_EACH _Pragma("unroll") for (int x = 0; x < N; ++x)
+    if (c.kmode == 1) {
+        MCD_EACH dv[x] = (T)0, K[x] = c.Kc;
+        return;
+    }
     MCD_EACH
     {
         const T dm = fabsf(__fadd_rn(__fsub_rn(u[x].mh, v[x].mh), __fsub_rn(u[x].ml, v[x].ml)));
@@ -314,8 +324,7 @@ __device__ __forceinline__ void pair_flat(const PairK<float> &c, bool early, con
     MCD_EACH
     {
         const T s2 = __fadd_rn(u[x].a, v[x].a);
-        K[x] = c.kmode == 1 ? c.Kc : __fmul_rn(__fmul_rn(__fmul_rn(c.pi, s2), s2), dv[x]);
-        dv[x] = c.kmode == 1 ? 0.0f : dv[x];
+        K[x] = __fmul_rn(__fmul_rn(__fmul_rn(c.pi, s2), s2), dv[x]);
     }
 #undef MCD_EACH
 }
