@@ -292,6 +292,7 @@ struct ClassLaunch {
     size_t smem;
     int ws, pl;  // the control-warp variant and its swarms per control lane
     int chain;   // the chain variant: nthr threads own swarms, and three more warps run beside them
+    int cols;    // the mixed chain without a matrix: columns of the first build kept in shared memory
 };
 
 // whether class k runs the control-warp variant: MCD_MIXED without the exact
@@ -315,6 +316,7 @@ static ClassLaunch class_launch(const CollideClass &k, int threads, int spt, int
     L.ws = ws;
     L.pl = ws ? ws_pl(k.n_hi) : 0;
     L.chain = 0;
+    L.cols = 0;
     if (ws) {
         L.S = 1;
         L.store = usable_store<T>(k, dv_matrix >= 0 ? dv_matrix : k.store);
@@ -351,7 +353,17 @@ static ClassLaunch class_launch(const CollideClass &k, int threads, int spt, int
     // exclusive: request more than half an SM's shared memory so that no two
     // collide CTAs of classes that can carry long chains share an SM (the
     // heaviest cells, launched first, run alone)
-    if (exclusive && k.n_hi > 64 && L.smem < kExclusiveSmem) L.smem = kExclusiveSmem;
+    if (exclusive && k.n_hi > 64 && L.smem < kExclusiveSmem) {
+        // (mixed chain without a matrix: the warps that own no swarm form their share of
+        // the first build's columns into the memory that is left)
+        if (sizeof(T) == 4 && L.chain && L.store == 0) {
+            const int warps = chain_build_warps(L.nthr), idle = std::max(warps - (k.n_hi + 31) / 32, 0);
+            const size_t col = (size_t)L.nthr * sizeof(float), room = ((size_t)smem_optin - L.smem) / col;
+            L.cols = (int)std::min<size_t>(room, (size_t)k.n_hi * idle / warps);
+            L.smem += L.cols * col;
+        }
+        L.smem = std::max(L.smem, kExclusiveSmem);
+    }
     return L;
 }
 
@@ -451,6 +463,7 @@ static cudaError_t collide_impl(mcd_ctx *cx, int from_state, double t_end)
         A.dv_w = k.W;
         A.dv_rows = k.rows;
         A.early = k.smem_fits;
+        A.cols = L.cols;
         A.dvg = L.store == 2 ? k.dvg : nullptr;
         unsigned grid = (unsigned)k.cells;
         A.qhead = nullptr;
@@ -638,7 +651,8 @@ static cudaError_t tune_impl(mcd_ctx *c)
                                                   c->exact_total, c->smem_optin, cs.ws);
             if (L.S != cs.S || L.store != cs.store) continue;  // (the launch would not run this candidate)
             if (L.smem > (size_t)c->smem_optin) continue;
-                A.dvg = L.store == 2 ? k.dvg : nullptr;
+            A.cols = L.cols;
+            A.dvg = L.store == 2 ? k.dvg : nullptr;
             float ms[kTrialRuns + 1] = {};
             for (int rep = 0; rep <= kTrialRuns && e == cudaSuccess; ++rep) {
                 e = cudaMemcpyAsync(A.m, c->m[b], 8 * c->N, cudaMemcpyDeviceToDevice, st);

@@ -780,6 +780,7 @@ struct CollideArgs {
     int dv_w;         // row width of the stored matrix (STORE)
     int early;        // chain variants: the class's matrix fits in shared memory (pair_flat)
     int dv_rows;      // rows per cell of the stored matrix (the class's largest cell)
+    int cols;         // chain variants without a stored matrix: columns of the first build that shared memory holds
     double *q;        // the tracer column (TRACER variants)
     void *dvg;        // STORE == 2: the class's matrices in the workspace, dv_rows x dv_w entries of T per queue entry
 };

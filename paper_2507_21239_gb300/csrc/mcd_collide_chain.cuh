@@ -92,6 +92,7 @@ struct ChainShared {
     alignas(8) float2 at;          // a choice: the prefix below the bracketing group, and that group (as an int)
     alignas(8) int2 sel;           // x: i, -2 at the end; y: the fresh R_i of the last event's swarm (as a float)
     alignas(8) int2 pick;          // x: which of the ready outcomes (-1: no partner bracketed, -2: the end), y: the event crosses t_end
+    int none;                      // MB > 1: the first waiting time is beyond t_end
     int ticket;                    // persistent CTAs: the queue entry taken
 };
 
@@ -262,7 +263,9 @@ __device__ __forceinline__ Part<float> make_part_rn(const CellK<float> &c, doubl
 // with early set, a pair of two swarms that no event of this chain has renewed
 // takes the drift and settling terms' sum with the other product fused, the
 // rounding in which a stored matrix's first build forms it.
-template <int N, bool EARLY>
+// COMMON (the first row sums, where a whole warp agrees): no v is a Stokes-law swarm,
+// no pair in turbulence regime I and no swarm renewed, so a fifth of the terms is left out.
+template <int N, bool EARLY, bool COMMON = false>
 __device__ __forceinline__ void pair_flat(const PairK<float> &c, bool early, const Part<float> (&u)[N],
                                           const Part<float> (&v)[N], float (&dv)[N], float (&K)[N])
 {
@@ -283,8 +286,9 @@ __device__ __forceinline__ void pair_flat(const PairK<float> &c, bool early, con
     {
         S1[x] = fmaxf(u[x].S, v[x].S), S2[x] = fminf(u[x].S, v[x].S);
         s[x] = __fadd_rn(S1[x], S2[x]);
-        g1[x] = __fmul_rn(__fmul_rn(c.vg2, __fmaf_rn(S1[x], S2[x], __fmul_rn(c.Se, s[x]))),
-                          rcp_ftz(__fmul_rn(__fmul_rn(s[x], __fadd_rn(S1[x], c.Se)), __fadd_rn(S2[x], c.Se))));
+        if (!COMMON)
+            g1[x] = __fmul_rn(__fmul_rn(c.vg2, __fmaf_rn(S1[x], S2[x], __fmul_rn(c.Se, s[x]))),
+                              rcp_ftz(__fmul_rn(__fmul_rn(s[x], __fadd_rn(S1[x], c.Se)), __fadd_rn(S2[x], c.Se))));
     }
     MCD_EACH
     {
@@ -297,8 +301,8 @@ __device__ __forceinline__ void pair_flat(const PairK<float> &c, bool early, con
     }
     MCD_EACH
     {
-        const bool su = u[x].fl & 4, sv = v[x].fl & 4;
-        const T as = su ? u[x].a : v[x].a, ads = su ? u[x].ad : v[x].ad;
+        const bool su = u[x].fl & 4, sv = !COMMON && (v[x].fl & 4);
+        const T as = su || COMMON ? u[x].a : v[x].a, ads = su || COMMON ? u[x].ad : v[x].ad;
         const T D_st = __fmul_rn(__fmul_rn(c.Cst, __fadd_rn(u[x].a, v[x].a)), da[x]);
         const T D_mx = __fmul_rn(c.Cst, __fmaf_rn(as, ads, __fmul_rn(c.asw, da[x]))), D_ep = __fmul_rn(c.Cep, da[x]);
         D[x] = (su && sv) ? D_st : ((su || sv) ? D_mx : D_ep);
@@ -312,8 +316,8 @@ __device__ __forceinline__ void pair_flat(const PairK<float> &c, bool early, con
         const T qv = __fmul_rn(u[x].q, v[x].q), qq = c.settle ? __fmul_rn(qv, qv) : 1.0f;
         const T Y = __fmaf_rn(__fmul_rn(c.e1, s[x]), s[x], __fmul_rn(__fmul_rn(c.e4, om), om)), pp2 = __fmul_rn(pp, pp);
         T Z = __fmaf_rn(c.oz2, qq, __fmul_rn(pp2, Y));
-        if (EARLY && early && !((u[x].fl | v[x].fl) & kFlRenewed)) Z = __fmaf_rn(pp2, Y, __fmul_rn(c.oz2, qq));
-        coef[x] = __fadd_rn(Z, (cls == 0 && s[x] > 0.0f) ? g1[x] : 0.0f);
+        if (EARLY && early && (COMMON || !((u[x].fl | v[x].fl) & kFlRenewed))) Z = __fmaf_rn(pp2, Y, __fmul_rn(c.oz2, qq));
+        coef[x] = COMMON ? Z : __fadd_rn(Z, (cls == 0 && s[x] > 0.0f) ? g1[x] : 0.0f);
         t0[x] = __fmaf_rn(c.cbm, __fadd_rn(u[x].im, v[x].im), cls == 1 ? t2[x] : (cls == 2 ? t3[x] : 0.0f));
     }
     MCD_EACH
@@ -354,6 +358,10 @@ inline size_t collide_chain_smem_bytes(int nsl, bool tracer, int store, int rows
     if (store == 1) b += (size_t)rows * W * sizeof(float);
     return b;
 }
+
+// warps that share the first row sums of a chain launch without a stored matrix: a
+// multiple of four, one sub-partition's worth over that would wait for the others
+__host__ __device__ inline int chain_build_warps(int nsl) { return (nsl / 32 + kChainRoles) & ~3; }
 
 // a swarm's cache or another's, field by field (no branch)
 __device__ __forceinline__ Part<float> part_select(bool other, const Part<float> &o, const Part<float> &p)
@@ -420,7 +428,7 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
     T *xs = rn + RW;                                                 // the scans' rows             
     T *pf = xs + 4 * nsl;                                      // prefixes within the groups
     T *dvrow = pf + nsl;                                             // dv of row i
-    T *Dm = dvrow + nsl;                                             // STORE == 1
+    T *Dm = dvrow + nsl;                                             // STORE == 1 (0: the first build's columns)
     const int W = A.dv_w;
     if constexpr (STORE == 2) Dm = reinterpret_cast<T *>(A.dvg) + (size_t)entry * A.dv_rows * W;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -468,14 +476,6 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
             if (TRACER) qsh[k] = A.q[off + k];
             parts[k] = pk;
         }
-        for (int e = 0; e < 2; ++e) {
-            const double mr = ready_mass(c, mk, dmm, e != 0);
-            const Part<T> pr = make_part_rn(c, mr, pk.Mv, kFlRenewed);
-            if (act) {
-                ready[e * nsl + k] = pr;
-                mready[e * nsl + k] = make_double2(mr, __dmul_rn(c.dm, mr));
-            }
-        }
     }
     __syncthreads();
 
@@ -485,26 +485,142 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
     int64_t ev = 0;
 
     const bool early = A.early != 0;
+    T *const xw = xs + 128 * w;
+    Acc<T> R;
+    R.zero();
+    // row sums R_k += r_kj in j order, two at a time: from the stored matrix, from
+    // columns formed by the warps that own no swarm, or from fresh entries (the same bits)
+    auto add_stored = [&](int j0, int j1) {
+        const int kc = act ? k : n - 1;
+#pragma unroll 4
+        for (int j = j0; j < j1; ++j) {
+            const Part<T> pj = parts[j];
+            const T dv = STORE != 0 ? Dm[sym_at(kc, j, n, W)] : Dm[(j - j0) * nsl + k];
+            R.add(kern_of<T>(pc, pk.a, pj.a, dv) * weight<T>(pk, pj));
+        }
+    };
+    auto fresh2 = [&](const Part<T> (&u)[2], const Part<T> (&o)[2], T (&dv)[2], T (&K)[2], bool first) {
+        const int fl = min(o[0].fl & 3, o[1].fl & 3);
+        if (first && fl && !((o[0].fl | o[1].fl) & 4))
+            pair_flat<2, true, true>(pc, early, u, o, dv, K);
+        else
+            pair_flat<2, true>(pc, early, u, o, dv, K);
+    };
+    auto add_fresh = [&](int j0, int j1, bool first) {
+        const Part<T> u[2] = {pk, pk};
+        for (int j = j0; j < j1; j += 2) {
+            const Part<T> o[2] = {parts[j], parts[min(j + 1, n - 1)]};
+            T dv[2], K[2];
+            fresh2(u, o, dv, K, first);
+            R.add(K[0] * weight<T>(pk, o[0]));
+            if (j + 1 < j1) R.add(K[1] * weight<T>(pk, o[1]));
+        }
+    };
+    const bool swarms = 32 * w < n;  // (a worker warp with swarms)
     if constexpr (STORE != 0) {
-        // every unordered pair once (warp w takes rows w, w + ng + 3, ...; its lanes
-        // consecutive offsets d, so the stores are consecutive words), two at a time
-        for (int rr = w; rr < n; rr += ng + kChainRoles) {
-            const Part<T> pr[2] = {parts[rr], parts[rr]};
-            const int dmax = (n - 1) / 2 + (((n & 1) == 0 && rr < n / 2) ? 1 : 0);
-            for (int d = lane; d <= dmax; d += 64) {
-                const int d2 = min(d + 32, dmax);
-                int j = rr + d, j2 = rr + d2;
-                if (j >= n) j -= n;
-                if (j2 >= n) j2 -= n;
-                const Part<T> pj[2] = {parts[j], parts[j2]};
-                T dv[2], K[2];
+        // every unordered pair once, in row order over all the CTA's threads (a row of a
+        // small cell fills no warp), two at a time: pair t is offset t mod L of row t / L,
+        // and the pairs half an even cell apart follow
+        const int L = (n - 1) / 2 + 1, half = (n & 1) ? 0 : n / 2, pairs = n * L + half;
+        const int step_r = nthr / L, step_d = nthr - step_r * L;
+        int rr = tid / L, d = tid - rr * L, t = tid;
+        while ((MB == 1 ? t - lane : t) < pairs) {  // (whole warps, where they vote)
+            int row[2], other[2], at2[2];
+            bool in[2];
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {
+                in[x] = t < pairs;
+                row[x] = !in[x] ? 0 : (t < n * L ? rr : t - n * L);
+                const int o = !in[x] ? 0 : (t < n * L ? d : half);
+                at2[x] = row[x] * W + o;
+                other[x] = row[x] + o;
+                if (other[x] >= n) other[x] -= n;
+                t += nthr, rr += step_r, d += step_d;
+                if (d >= L) d -= L, ++rr;
+            }
+            const Part<T> pr[2] = {parts[row[0]], parts[row[1]]}, pj[2] = {parts[other[0]], parts[other[1]]};
+            T dv[2], K[2];
+            // (with several CTAs per SM the second form's registers would be spilled ones)
+            const int cls = min(max(pr[0].fl & 3, pj[0].fl & 3), max(pr[1].fl & 3, pj[1].fl & 3));
+            if (MB == 1 && __all_sync(0xffffffffu, cls && !((pj[0].fl | pj[1].fl) & 4)))
+                pair_flat<2, true, true>(pc, early, pr, pj, dv, K);
+            else
                 pair_flat<2, true>(pc, early, pr, pj, dv, K);
-                Dm[rr * W + d] = dv[0];
-                if (d + 32 <= dmax) Dm[rr * W + d2] = dv[1];
+            if (MB > 1 || in[0]) Dm[at2[0]] = dv[0];
+            if (in[1]) Dm[at2[1]] = dv[1];
+        }
+        __syncthreads();
+        if (swarms) add_stored(0, n);
+    } else {
+        // the last columns by the warps without swarms, the others by their owners
+        // (as many of them as leave every SM sub-partition the same number of warps).  4,096
+        // cells of 300 swarms, collide of a 0.1-yr step: 2,004 -> 1,772 us, of 400: 3,187 ->
+        // 2,650, with the terms that COMMON leaves out (the block kernel's shared half
+        // matrix: 1,789; 400 swarms recomputing: 3,210).
+        const int warps = chain_build_warps(nsl), busy = (n + 31) >> 5, idle = max(warps - busy, 0);
+        const int cols = min(A.cols, n * idle / warps) & ~1, j0 = n - cols;
+        if (swarms) {
+            add_fresh(0, j0, true);
+        } else if (w - busy < idle) {
+            for (int j = j0 + 2 * (w - busy); j < n; j += 2 * idle) {
+                const Part<T> o[2] = {parts[j], parts[j + 1]};
+                for (int q = lane; q < 32 * busy; q += 32) {
+                    const Part<T> u[2] = {parts[min(q, n - 1)], parts[min(q, n - 1)]};
+                    T dv[2], K[2];
+                    fresh2(u, o, dv, K, true);
+                    Dm[(j - j0) * nsl + q] = dv[0];
+                    Dm[(j + 1 - j0) * nsl + q] = dv[1];
+                }
+            }
+        }
+        __syncthreads();
+        if (swarms) add_stored(j0, n);
+    }
+    T hi = act ? (T)R.hi() : (T)0;  // R_k for the next choice
+    if constexpr (MB > 1) {
+        // The first waiting time: most of many light cells have no event in a short step,
+        // and need neither ready outcomes nor choices.  32,768 cells of 32 swarms, collide
+        // of a 0.001-yr step (no events) 485 -> 279 us with the pairs above in row order,
+        // of a 0.1-yr one 557 -> 371 (block-wide scans: 293, 342; with more events than
+        // 0.4 per cell the chain is ahead: 1 yr 2,103 -> 1,724).  In the one-CTA kernels the
+        // ready outcomes are 3 % of a cell, and the branch costs the event loop as much.
+        if (w < ng) {
+            const T x = group_prefix(xw, hi);
+            if (lane == 31) sh.ti[2 * NW - ng + w] = x;
+        }
+        __syncthreads();
+        if (w == ng + 1) {
+            T all[NW];
+            load_words<NW>(sh.ti + NW, all);
+            const T tot = tree_down<NW>(all);
+            const double t_end = A.t_end_from_state ? A.state->t + A.state->dt : A.t_end_fixed;
+            const bool none = tot > (T)0 && A.max_events > 0 && A.state->t + (double)fdiv(sh.ring[0].L, tot) >= t_end;
+            if (lane == 0) {
+                sh.none = none;
+                if (none) {
+                    A.cell_events[cell] = 0;
+                    if (cell == A.log_cell) *A.log_n = 0;
+                    if (A.Rtot) A.Rtot[cell] = (double)tot / c.sc;
+                }
+            }
+        }
+        __syncthreads();
+        if (sh.none) {
+            if (act && A.Rdump) A.Rdump[off + k] = R.value() / c.sc;
+            return;
+        }
+    }
+    if (w < ng) {
+        const double2 mk = mm[act ? k : n - 1];
+        for (int e = 0; e < 2; ++e) {
+            const double mr = ready_mass(c, mk.x, mk.y, e != 0);
+            const Part<T> pr = make_part_rn(c, mr, pk.Mv, kFlRenewed);
+            if (act) {
+                ready[e * nsl + k] = pr;
+                mready[e * nsl + k] = make_double2(mr, __dmul_rn(c.dm, mr));
             }
         }
     }
-    __syncthreads();
 
     if (w == ng) {  // ---- the choice warp ----
         const bool logging = (cell == A.log_cell);
@@ -676,37 +792,12 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
         }
     } else {  // ---- the workers ----
         int pend = -1;  // swarm whose fresh row sum rides on the next choice
-        Acc<T> R;
-        // full build of the row sums: R_k = sum_j r_kj in j order, from the stored
-        // matrix or from fresh entries two at a time
-        auto build = [&]() {
-            R.zero();
-            if constexpr (STORE != 0) {
-                const int kc = act ? k : n - 1;
-#pragma unroll 4
-                for (int j = 0; j < n; ++j) {
-                    const Part<T> pj = parts[j];
-                    R.add(kern_of<T>(pc, pk.a, pj.a, Dm[sym_at(kc, j, n, W)]) * weight<T>(pk, pj));
-                }
-            } else {
-                const Part<T> u[2] = {pk, pk};
-                for (int j = 0; j < n; j += 2) {
-                    const Part<T> o[2] = {parts[j], parts[min(j + 1, n - 1)]};
-                    T dv[2], K[2];
-                    pair_flat<2, true>(pc, early, u, o, dv, K);
-                    R.add(K[0] * weight<T>(pk, o[0]));
-                    if (j + 1 < n) R.add(K[1] * weight<T>(pk, o[1]));
-                }
-            }
-        };
-        build();
         bar_arrive(kBarNew, nsl + 32);
-        T *const xw = xs + 128 * w;
         int guess = 0;  // the kind of ready outcome that came last
-        // R_k for the next choice (0 for the swarm whose fresh sum rides on it), and
-        // what is put off until the choice is under way: the event's entry of the
+        // hi is 0 for the swarm whose fresh sum rides on the next choice; what is put off
+        // until the choice is under way: the event's entry of the
         // matrix, the updated R_k, and (took) the swarm's own new cache
-        T hi = act ? (T)R.hi() : (T)0, dvn = (T)0;
+        T dvn = (T)0;
         Acc<T> Rn = R;
         Part<T> us = pk;
         bool upd = false, took = false;
@@ -799,7 +890,9 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
                 took = false;
                 if (STORE != 0 && act) Dm[at] = dvn;
                 bar_sync(kBarBuild, nsl + 32);
-                build();
+                R.zero();
+                if (swarms && STORE != 0) add_stored(0, n);
+                if (swarms && STORE == 0) add_fresh(0, n, false);
                 Rn = R;
                 pend = -1;
                 until_rebuild = reb;
