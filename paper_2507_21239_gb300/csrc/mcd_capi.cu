@@ -274,6 +274,7 @@ int mcd_init_disk(mcd_ctx **out, const mcd_disk_params *p, const mcd_grid *g, in
         for (int64_t k = 0; k < (int64_t)D.n_r * D.n_z; ++k) cell_disk[D.c_off + k] = d;
         for (int64_t k = 0; k < D.n_r; ++k) zone_disk[D.z_off + k] = d;
         for (int64_t k = 0; k < D.n_tiles; ++k) tile_disk[D.t_off + k] = d;
+        c->sup_rows += (int64_t)D.n_tiles * ((D.n_tiles + kRadixGroup - 1) / kRadixGroup);
         for (int64_t k = 0; k < D.n0; ++k) slot_disk[D.p_off + k] = d;
         Msw[d] = disk_dust_mass(p[d]) / (double)D.n0;
     }

@@ -290,7 +290,7 @@ constexpr int kRunShortMax = 64;
 constexpr int kRadixThreads = 256, kRadixItems = 8, kRadixTile = kRadixThreads * kRadixItems;
 constexpr int kRadixBins = 256, kRadixPasses = 8;
 constexpr int kRadixGroup = 16;   // tiles per group (a disk's start at sup_off)
-constexpr int kRadixDirect = 64;  // groups a scatter CTA adds up itself
+constexpr int64_t kRadixDirectRows = 65536;  // group rows that a pass's scatter CTAs add up themselves
 constexpr int kRadixUpperPasses = 4;  // the r sort runs the passes of the keys' upper four bytes
 // A disk's first group: floor(t_off / 16) + its number leaves every disk room for
 // its last, partly filled group; n_sup is the end of the last disk's.
@@ -352,6 +352,7 @@ struct mcd_ctx {
     int64_t N = 0, C = 0, Z = 0, n_tiles = 0;
     int32_t n_max = 0;  // largest possible cell population
     int64_t zone_max = 0, n0_max = 0;  // largest radial zone (n_z * per_cell) and disk (particles)
+    int64_t sup_rows = 0;              // the disks' radix tiles times groups of tiles
 
     mcd_disk_params *d_params = nullptr;
     mcd::DiskC<float> *d_cf = nullptr;   // per disk: transport's constants (MCD_MIXED)

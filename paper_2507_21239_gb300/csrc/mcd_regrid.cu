@@ -135,10 +135,11 @@ __device__ __forceinline__ uint32_t digit_excl_scan(uint32_t x, uint32_t *wsum)
 
 // Large disks: one CTA per disk turns the groups' counts into their first
 // destination per digit, so that a scatter CTA reads one row instead of all.
-// Up to kRadixDirect groups (2,097,152 particles) a CTA adds them up itself, a
-// launch less per pass; a regrid added up / scanned: 65,536 particles 85 / 101
-// us, 819,200 146 / 156, 1,638,400 (50 groups) 258 / 270, 3,276,800 (100
-// groups) 790 / 767.
+// Up to kRadixDirectRows rows in all (tiles times groups; one disk of 2,097,152
+// particles) a CTA adds up its disk's groups itself, a launch less per pass; a
+// regrid added up / scanned: 65,536 particles 85 / 101 us, 819,200 146 / 156,
+// 1,638,400 (40,000) 258 / 270, 3,276,800 (160,000) 790 / 767, 64 disks of
+// 28.5 M particles (290,000) 3,504 / 3,352.
 constexpr int kSupSlices = 4;  // a disk's groups in four slices: the loads are what it waits for
 
 __global__ void __launch_bounds__(kSupSlices *kRadixBins) k_sup_scan(const DiskDev *disks, uint32_t *sup)
@@ -821,8 +822,7 @@ cudaError_t launch_regrid(mcd_ctx *c)
     const int64_t nsup = c->n_sup * kRadixBins;
     k_regrid_keys<<<gN, 256, 0, st>>>(c->d_disks, c->slot_disk, c->N, c->r[b], c->z[b], c->id[b], c->key[0],
                                       c->val[0], c->status, c->sup, nsup * kRadixUpperPasses, c->rfix_count);
-    const int64_t groups_max = (c->n0_max + (int64_t)kRadixTile * kRadixGroup - 1) / ((int64_t)kRadixTile * kRadixGroup);
-    const int scanned = groups_max > kRadixDirect;
+    const int scanned = c->sup_rows > kRadixDirectRows;
     // the upper four bytes of the keys (an even number of passes: the result is back in buffer 0)
     for (int pass = kRadixPasses - kRadixUpperPasses; pass < kRadixPasses; ++pass) {
         const int shift = 8 * pass, src = pass & 1, dst = src ^ 1;
