@@ -158,7 +158,7 @@ static int block_threads(int swarm_threads, bool exact)
 static bool smem_matrix_fits(int n)
 {
     for (int S = 1; S <= 2; ++S)
-        if (collide_smem_bytes<float>(class_threads(n, S), S, true, 1, n, sym_width(n), false) + kStaticReserve >
+        if (collide_smem_bytes(class_threads(n, S), S, true, 1, n, sym_width(n), false) + kStaticReserve >
             kSmemOptinMax)
             return false;
     return true;
@@ -217,19 +217,15 @@ int plan_classes(const mcd_grid *g, int32_t nd, int32_t prec, std::vector<Collid
 }
 
 // ---- launches ------------------------------------------------------------------------
-template <class T>
+// the block kernels (mixed precision)
 static cudaError_t variant(int op, int S, int store, bool ramp, bool tracer, bool exact, unsigned grid, int nthr,
                            size_t smem, cudaStream_t st, const CollideArgs *A, int *out)
 {
-    if constexpr (sizeof(T) == 8) {
-        return cudaErrorInvalidValue;  // (FP64 launches are chain launches)
-    } else {
-        if (exact)
-            return S == 2 ? collide_variant<float, 2, true>(op, store, ramp, tracer, grid, nthr, smem, st, A, out)
-                          : collide_variant<float, 1, true>(op, store, ramp, tracer, grid, nthr, smem, st, A, out);
-        return S == 2 ? collide_variant<float, 2, false>(op, store, ramp, tracer, grid, nthr, smem, st, A, out)
-                      : collide_variant<float, 1, false>(op, store, ramp, tracer, grid, nthr, smem, st, A, out);
-    }
+    if (exact)
+        return S == 2 ? collide_variant<2, true>(op, store, ramp, tracer, grid, nthr, smem, st, A, out)
+                      : collide_variant<1, true>(op, store, ramp, tracer, grid, nthr, smem, st, A, out);
+    return S == 2 ? collide_variant<2, false>(op, store, ramp, tracer, grid, nthr, smem, st, A, out)
+                  : collide_variant<1, false>(op, store, ramp, tracer, grid, nthr, smem, st, A, out);
 }
 
 // the chain variants for launches of nsl swarm slots
@@ -338,7 +334,7 @@ static ClassLaunch class_launch(const CollideClass &k, int threads, int spt, int
     auto bytes = [&]() {
         if (sizeof(T) == 8) return collide_chain64_smem_bytes(L.nthr, tracer != 0);
         return L.chain ? collide_chain_smem_bytes(L.nthr, tracer != 0, L.store, k.rows, k.W)
-                       : collide_smem_bytes<T>(L.nthr, L.S, tracer != 0, L.store, k.rows, k.W, exact);
+                       : collide_smem_bytes(L.nthr, L.S, tracer != 0, L.store, k.rows, k.W, exact);
     };
     L.smem = bytes();
     if (L.chain && L.store == 1 && L.smem > (size_t)smem_optin) {  // (no room beside the ready outcomes)
@@ -390,7 +386,7 @@ static cudaError_t launch_op(int op, const ClassLaunch &L, bool ramp, bool trace
 {
     if (L.chain) return chain_variant<T>(op, L.nthr, L.store, ramp, tracer, grid, L.smem, st, A, out);
     if (L.ws) return ws_variant(op, L.pl, L.store, ramp, tracer, grid, L.nthr, L.smem, st, A, out);
-    return variant<T>(op, L.S, L.store, ramp, tracer, exact, grid, L.nthr, L.smem, st, A, out);
+    return variant(op, L.S, L.store, ramp, tracer, exact, grid, L.nthr, L.smem, st, A, out);
 }
 
 template <class T>
@@ -502,11 +498,11 @@ static cudaError_t prepare_impl(mcd_ctx *c)
             for (int store = 0; store <= 2; ++store) {
                 if (S == 1 && !exact && store != 1) continue;  // (the chain variants, below)
                 int st = 0;
-                if ((e = variant<T>(2, S, store, false, false, exact, 0, 0, 0, nullptr, nullptr, &st)) != cudaSuccess)
+                if ((e = variant(2, S, store, false, false, exact, 0, 0, 0, nullptr, nullptr, &st)) != cudaSuccess)
                     return e;
                 const int dyn = optin - st;
                 if (dyn <= 0) return cudaErrorInvalidValue;
-                if ((e = variant<T>(1, S, store, false, false, exact, 0, 0, (size_t)dyn, nullptr, nullptr,
+                if ((e = variant(1, S, store, false, false, exact, 0, 0, (size_t)dyn, nullptr, nullptr,
                                     nullptr)) != cudaSuccess)
                     return e;
                 smin = std::min(smin, dyn);

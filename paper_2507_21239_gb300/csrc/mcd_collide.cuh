@@ -6,7 +6,13 @@
 // from R_tot = sum_i R_i, i chosen by R_i and j by r_ij, and only row and
 // column i change after an event.
 //
-// GB300 layout: one CTA per cell, S swarms per thread (S = 1 or 2; swarm k is
+// This file holds what every collide kernel shares (caches, pair entries, outcomes)
+// and the block kernels, mixed precision with two swarms per thread, with the
+// compensated total rate, or with a shared matrix that leaves the chain kernels no
+// room; the chain kernels (mcd_collide_chain.cuh, mcd_collide_chain64.cuh for FP64)
+// run everything else.
+//
+// The block kernels: one CTA per cell, S swarms per thread (S = 1 or 2; swarm k is
 // owned by thread k / S).  The per-swarm cache (radius, Stokes number,
 // drag-law flags, 1/m, M/V, ...) sits in shared memory; each thread keeps the
 // row sums R_k of its swarms in registers.  The per-cell gas constants come
@@ -26,7 +32,7 @@
 // memory (FP32, when it fits) or in the workspace (FP64; FP32 for cells too
 // large for shared memory).
 //
-// Precision (template T): T = double is the plain FP64 path.  T = float is
+// Precision (template T of the shared parts): T = double is the FP64 path, T = float
 // the mixed path: dv, sigma, K, rates, waiting times and partner choice in
 // FP32; masses and the cell clock in FP64 (touched by one lane per event,
 // because an FP64 instruction costs ~64 cycles on GB300); row sums R_k as
@@ -44,8 +50,6 @@
 #pragma once
 #include <float.h>
 #include <math.h>
-
-#include <type_traits>
 
 #include "mcd_internal.cuh"
 
@@ -483,19 +487,12 @@ __device__ __forceinline__ int sym_at(int i, int j, int n, int W)
 // brackets the target and finds the thread by a ballot (and the element
 // within the thread from the previous thread's prefix).  block_bracket returns
 // the element in that warp's lane 0 and -1 in every other lane (one barrier).
-// A passive warp (no elements) skips its own scan.  FP64 comparisons go through
-// the bit patterns (prefixes of rates are not negative).
-__device__ __forceinline__ bool lt_rate(float a, float b) { return a < b; }
-__device__ __forceinline__ bool lt_rate(double a, double b) { return __double_as_longlong(a) < __double_as_longlong(b); }
-__device__ __forceinline__ bool finite_rate(float a) { return true; }  // (its comparisons see a NaN themselves)
-__device__ __forceinline__ bool finite_rate(double a)
+// A passive warp (no elements) skips its own scan.
+template <int S, bool FUSE>
+__device__ __forceinline__ int block_bracket(const float (&x)[S], const float (&y)[S], float u, int pend, float *buf,
+                                             float &total, float &ysum, bool passive = false)
 {
-    return ((unsigned)(__double_as_longlong(a) >> 52) & 0x7FFu) != 0x7FFu;
-}
-template <class V, int S, bool FUSE>
-__device__ __forceinline__ int block_bracket(const V (&x)[S], const V (&y)[S], V u, int pend, V *buf, V &total,
-                                             V &ysum, bool passive = false)
-{
+    typedef float V;
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     V wi = x[0], ys = FUSE ? y[0] : (V)0;
@@ -535,12 +532,12 @@ __device__ __forceinline__ int block_bracket(const V (&x)[S], const V (&y)[S], V
     total = tot + Rp;
     ysum = Rp;
     V target = u * total;
-    if (!lt_rate(target, total)) target = total * (V)(1.0 - 1e-7);
+    if (!(target < total)) target = total * (V)(1.0 - 1e-7);
     const int e0 = S * (int)threadIdx.x;
     const V P = (off + wi) + ((pend >= 0 && e0 + S - 1 >= pend) ? Rp : (V)0);
     const V lo = off + ((pend >= 0 && S * 32 * w > pend) ? Rp : (V)0);
     const V hi = hib + ((pend >= 0 && S * 32 * (w + 1) - 1 >= pend) ? Rp : (V)0);
-    const unsigned bal = __ballot_sync(FULL, lt_rate(target, P));
+    const unsigned bal = __ballot_sync(FULL, target < P);
     // (a tree scan may leave lane 31's prefix an ulp below hi: then lane 31)
     const int l = __ffs(bal | 0x80000000u) - 1;
     int sub = 0;
@@ -562,7 +559,7 @@ __device__ __forceinline__ int block_bracket(const V (&x)[S], const V (&y)[S], V
         }
         sub = __shfl_sync(FULL, first >= 0 ? first : last, l);
     }
-    return (lane == 0 && finite_rate(total) && !lt_rate(target, lo) && lt_rate(target, hi)) ? S * (32 * w + l) + sub : -1;
+    return (lane == 0 && !(target < lo) && target < hi) ? S * (32 * w + l) + sub : -1;
 }
 
 // ---- compensated FP32 sums ---------------------------------------------------------
@@ -699,7 +696,6 @@ struct Acc<double> {
     __device__ double hi() const { return s; }
     __device__ double value() const { return s; }
     __device__ void set(double x) { s = x; }
-    __device__ void set2(double h, double l) { s = h + l; }
 };
 template <>
 struct Acc<float> {
@@ -785,13 +781,12 @@ struct CollideArgs {
     void *dvg;        // STORE == 2: the class's matrices in the workspace, dv_rows x dv_w entries of T per queue entry
 };
 
-template <class T>
 struct Shared {
-    CellK<T> c;
-    T scan[2][64];
-    float tot_h, tot_e, y_h, y_e;  // FP32: the helper warp's compensated total rate and fresh row sum
+    CellK<float> c;
+    float scan[2][64];
+    float tot_h, tot_e, y_h, y_e;  // the helper warp's compensated total rate and fresh row sum
     int sel;
-    Draw<T> ring[32];
+    Draw<float> ring[32];
     double t;    // the cell clock
     int stop;    // 0 event applied, 1 crossing t_end, 2 no partner bracketed
     int ticket;  // persistent CTAs: the queue entry taken
@@ -803,16 +798,17 @@ struct Shared {
 // on every event.  RAMP: a fragmentation probability ramp below v_frag.
 // entry: the cell's position in this launch's queue, which also picks its
 // slot of the launch's workspace matrices (STORE == 2; rebuilt at every start)
-template <class T, int S, int STORE, bool RAMP, bool TRACER, bool EXACT>
-__device__ __forceinline__ void cell_chain(const CollideArgs &A, const int64_t cell, const int64_t entry,
-                                           Shared<T> &sh, unsigned char *smem_raw)
+template <int S, int STORE, bool RAMP, bool TRACER, bool EXACT>
+__device__ __forceinline__ void cell_chain(const CollideArgs &A, const int64_t cell, const int64_t entry, Shared &sh,
+                                           unsigned char *smem_raw)
 {
+    typedef float T;
     const int nslot = blockDim.x * S;
     Part<T> *parts = reinterpret_cast<Part<T> *>(smem_raw);
     double *msh = reinterpret_cast<double *>(parts + nslot);
     T *dvrow = reinterpret_cast<T *>(msh + nslot);
     double *qsh = reinterpret_cast<double *>(dvrow + nslot);  // TRACER
-    constexpr bool COMP = sizeof(T) == 4 && EXACT;
+    constexpr bool COMP = EXACT;
     // (exact total) every swarm's row sum (s, c) and new-row entry, posted for the helper warp
     float4 *post = reinterpret_cast<float4 *>(TRACER ? reinterpret_cast<unsigned char *>(qsh + nslot)
                                                      : reinterpret_cast<unsigned char *>(qsh));
@@ -822,7 +818,7 @@ __device__ __forceinline__ void cell_chain(const CollideArgs &A, const int64_t c
     if constexpr (STORE == 2) Dm = reinterpret_cast<T *>(A.dvg) + (size_t)entry * A.dv_rows * W;
     const int k0 = S * (int)threadIdx.x;  // this thread's first swarm
     const int lane = threadIdx.x & 31;
-    // FP32 with the compensated total (EXACT): the last warp holds no swarm; it
+    // with the compensated total (EXACT): the last warp holds no swarm; it
     // sums the posted row sums into the compensated total rate while the others
     // form row i
     constexpr bool comp = COMP;
@@ -841,11 +837,7 @@ __device__ __forceinline__ void cell_chain(const CollideArgs &A, const int64_t c
     if (threadIdx.x == 0) sh.c = *reinterpret_cast<const CellK<T> *>(A.cellk + cell * kCellKBytes);
     __syncthreads();
     const CellK<T> &c = sh.c;
-    // FP32: the entry constants in registers; FP64: read in place (register budget)
-    typedef typename std::conditional<sizeof(T) == 4, PairK<T>, const CellK<T> &>::type PK;
-    PK pc = [&]() -> PK {
-        if constexpr (sizeof(T) == 4) return pair_consts<T>(sh.c); else return sh.c;
-    }();
+    const PairK<T> pc = pair_consts<T>(sh.c);  // (in registers)
     bool act[S];
     Part<T> pk[S];
 #pragma unroll
@@ -854,9 +846,9 @@ __device__ __forceinline__ void cell_chain(const CollideArgs &A, const int64_t c
         act[s] = k < n;
         if (act[s]) {
             const double mk = A.m[off + k];
-            // FP32 path: every mass the event loop can reach lies between the
-            // monomer mass and the disk's dust mass, inside the split's range
-            if (sizeof(T) == 4 && !mass_splits(mk)) atomicOr(A.status, kStBadCell);
+            // every mass the event loop can reach lies between the monomer mass and
+            // the disk's dust mass, inside the split's range
+            if (!mass_splits(mk)) atomicOr(A.status, kStBadCell);
             msh[k] = mk;
             if (TRACER) qsh[k] = A.q[off + k];
             pk[s] = make_part<T>(c, mk, (T)(A.M[off + k] * c.invVsc));
@@ -905,8 +897,7 @@ __device__ __forceinline__ void cell_chain(const CollideArgs &A, const int64_t c
                 R[s].zero();
                 if (act[s]) {
                     int j = 0;
-                    // (FP64: no unrolling; its register budget is spent on the wider values)
-                    for (; sizeof(T) == 4 && j + 4 <= n; j += 4) {
+                    for (; j + 4 <= n; j += 4) {
                         T K0, K1, K2, K3;
                         const Part<T> p0 = parts[j], p1 = parts[j + 1], p2 = parts[j + 2], p3 = parts[j + 3];
                         pair_dv<T>(pc, pk[s], p0, &K0);
@@ -969,7 +960,7 @@ __device__ __forceinline__ void cell_chain(const CollideArgs &A, const int64_t c
         T tot, Rp;
         if (threadIdx.x == 0) sh.sel = -1;
         {
-            const int f = block_bracket<T, S, true>(val, rown, dr.u1, pend, sh.scan[0], tot, Rp, helper);
+            const int f = block_bracket<S, true>(val, rown, dr.u1, pend, sh.scan[0], tot, Rp, helper);
             if (f >= 0) sh.sel = f;
             __syncthreads();
         }
@@ -1046,12 +1037,11 @@ __device__ __forceinline__ void cell_chain(const CollideArgs &A, const int64_t c
         //     the clock and, unless the event would cross t_end (memoryless:
         //     discarded), applies the outcome and the new cache of i (FP64 masses)
         T tot2, unused;
-        int j = block_bracket<T, S, false>(row, zero, dr.u2, -1, sh.scan[1], tot2, unused, helper);
+        int j = block_bracket<S, false>(row, zero, dr.u2, -1, sh.scan[1], tot2, unused, helper);
         if (j >= 0) {
             if (j >= n) j = n - 1;  // (lane 31 fallback in a partly idle warp)
             // the clock, the outcome and the new cache are independent chains;
-            // only the stores wait for the crossing test.  FP32: the total rate
-            // is the helper warp's compensated sum
+            // only the stores wait for the crossing test
             T Rt = tot;
             if constexpr (COMP)
                 if (comp) Rt = __fadd_rn(sh.tot_h, sh.tot_e);
@@ -1150,11 +1140,11 @@ __device__ __forceinline__ void cell_chain(const CollideArgs &A, const int64_t c
 
 // One CTA per queue entry, or (qhead set) persistent CTAs that take entries
 // by an atomic ticket until the queue is exhausted.
-template <class T, int S, int STORE, bool RAMP, bool TRACER, bool EXACT>
+template <int S, int STORE, bool RAMP, bool TRACER, bool EXACT>
 __global__ void __launch_bounds__(kMaxCell / S) k_collide(CollideArgs A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ Shared<T> sh;
+    __shared__ Shared sh;
     int64_t entry = blockIdx.x;
     for (;;) {
         if (A.qhead) {
@@ -1165,21 +1155,20 @@ __global__ void __launch_bounds__(kMaxCell / S) k_collide(CollideArgs A)
         }
         if (entry >= A.n_queue) return;
         const int64_t cell = A.queue ? (int64_t)A.queue[entry] : entry;
-        cell_chain<T, S, STORE, RAMP, TRACER, EXACT>(A, cell, entry, sh, smem_raw);
+        cell_chain<S, STORE, RAMP, TRACER, EXACT>(A, cell, entry, sh, smem_raw);
         if (!A.qhead) return;
     }
 }
 
-// dynamic shared memory of a collide CTA of nthr threads (S swarms each):
-// caches, masses, the dv row, the tracer copy and (FP32, exact total) the
-// posted row sums; plus the stored matrix (STORE == 1) of rows x W entries
-template <class T>
+// dynamic shared memory of a block kernel's CTA of nthr threads (S swarms each):
+// caches, masses, the dv row, the tracer copy and (exact total) the posted row
+// sums; plus the stored matrix (STORE == 1) of rows x W entries
 inline size_t collide_smem_bytes(int nthr, int S, bool tracer, int store, int rows, int W, bool exact)
 {
     const size_t slots = (size_t)nthr * S;
-    size_t b = slots * (sizeof(Part<T>) + sizeof(double) + sizeof(T)) + (tracer ? slots * sizeof(double) : 0) +
-               (sizeof(T) == 4 && exact ? slots * sizeof(float4) : 0);
-    if (store == 1) b += (size_t)rows * W * sizeof(T);
+    size_t b = slots * (sizeof(Part<float>) + sizeof(double) + sizeof(float)) + (tracer ? slots * sizeof(double) : 0) +
+               (exact ? slots * sizeof(float4) : 0);
+    if (store == 1) b += (size_t)rows * W * sizeof(float);
     return b;
 }
 
@@ -1213,19 +1202,19 @@ inline cudaError_t variant_op(void (*const ks[4])(CollideArgs), int op, bool ram
     return e;
 }
 
-// the variants' host entry points, one translation unit per (T, S, EXACT);
-// ops as in variant_op
-template <class T, int S, bool EXACT>
+// the block kernels' host entry points, one translation unit per (S, EXACT); ops
+// as in variant_op
+template <int S, bool EXACT>
 cudaError_t collide_variant(int op, int store, bool ramp, bool tracer, unsigned grid, int nthr, size_t smem,
                             cudaStream_t st, const CollideArgs *A, int *out);
 
-template <class T, int S, int STORE, bool EXACT>
+template <int S, int STORE, bool EXACT>
 cudaError_t collide_variant_store(int op, bool ramp, bool tracer, unsigned grid, int nthr, size_t smem,
                                   cudaStream_t st, const CollideArgs *A, int *out)
 {
     void (*ks[4])(CollideArgs) = {
-        k_collide<T, S, STORE, false, false, EXACT>, k_collide<T, S, STORE, true, false, EXACT>,
-        k_collide<T, S, STORE, false, true, EXACT>, k_collide<T, S, STORE, true, true, EXACT>};
+        k_collide<S, STORE, false, false, EXACT>, k_collide<S, STORE, true, false, EXACT>,
+        k_collide<S, STORE, false, true, EXACT>, k_collide<S, STORE, true, true, EXACT>};
     return variant_op(ks, op, ramp, tracer, grid, nthr, smem, st, A, out);
 }
 

@@ -1,6 +1,6 @@
 // mcd_collide_chain.cuh -- the mixed-precision collision chain of one cell,
 // split over specialised warps.  Same method, same arithmetic and the same bits
-// as cell_chain<float, 1, ...> in mcd_collide.cuh would give (Zsom &
+// as cell_chain<1, ...> in mcd_collide.cuh would give (Zsom &
 // Dullemond's representative-particle scheme, Summary of the mcdust paper);
 // what differs is who does what between which barriers.
 //
@@ -37,13 +37,13 @@
 //    one Philox round per event.
 //
 // Measured, heaviest cell, us per event (one thread per swarm with block-wide
-// scans before -> now): 50 swarms 1.35 -> 0.84, 100: 1.40 -> 0.90, 200: 1.53 ->
-// 0.98, 300: 1.69 -> 1.33, 400: 1.97 -> 1.48, 500: 2.01 -> 1.62.  (Without the
+// scans before -> now): 50 swarms 1.35 -> 0.85, 100: 1.40 -> 0.91, 200: 1.53 ->
+// 0.98, 300: 1.69 -> 1.31, 400: 1.97 -> 1.47, 500: 2.01 -> 1.62.  (Without the
 // row sums formed ahead 0.93 at 100 and 1.03 at 200; with them 1.56 at 400,
 // where they compete with the choice for issue slots.)  Up to 256 swarms the
-// shared matrix beats recomputing row i (200 swarms: 0.98 against 1.14); where the ready outcomes leave no room for the matrix (from about 290)
-// recomputing in this layout beats the stored matrix in the block-scan layout
-// (1.33 against 1.69).  Two groups per worker warp, to issue what does not
+// shared matrix beats recomputing row i (200 swarms: 0.98 against 1.14); where the
+// ready outcomes leave no room for the matrix (from about 290) recomputing in this layout beats the stored matrix in the block-scan layout
+// (1.31 against 1.69).  Two groups per worker warp, to issue what does not
 // depend on the swarm once per sub-partition, were slower at every size (200:
 // 1.25, 400: 1.63): one warp's instructions issue in order, and two warps hide
 // each other's latencies where two streams in one do not.
@@ -261,8 +261,9 @@ __device__ __forceinline__ Part<float> make_part_rn(const CellK<float> &c, doubl
 // neither on the store nor on the warp that forms them; they are pair_dv's,
 // except that dv below 1e-19 cm/s (dv^2 no normal number) counts as 0.  EARLY:
 // with early set, a pair of two swarms that no event of this chain has renewed
-// takes the drift and settling terms' sum with the other product fused, the
-// rounding in which a stored matrix's first build forms it.
+// takes the drift and settling terms' sum with the other product fused.  Neither
+// rounding is the better one: it is kept so that runs of classes whose matrix fits
+// into shared memory (up to 318 swarms) give the bits they always gave.
 // COMMON (the first row sums, where a whole warp agrees): no v is a Stokes-law swarm,
 // no pair in turbulence regime I and no swarm renewed, so a fifth of the terms is left out.
 template <int N, bool EARLY, bool COMMON = false>
@@ -425,8 +426,8 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
     double2 *mready = mm + nsl;                                      // the same of ready
     double *qsh = reinterpret_cast<double *>(mready + 2 * nsl + 1);  // TRACER
     T *rn = reinterpret_cast<T *>(qsh + (TRACER ? nsl : 0));         // the last event's new row (zero beyond nsl)
-    T *xs = rn + RW;                                                 // the scans' rows             
-    T *pf = xs + 4 * nsl;                                      // prefixes within the groups
+    T *xs = rn + RW;                                                 // the scans' rows
+    T *pf = xs + 4 * nsl;                                            // prefixes within the groups
     T *dvrow = pf + nsl;                                             // dv of row i
     T *Dm = dvrow + nsl;                                             // STORE == 1 (0: the first build's columns)
     const int W = A.dv_w;

@@ -8,11 +8,11 @@
 namespace mcd {
 
 template <>
-cudaError_t collide_variant<float, 1, false>(int op, int store, bool ramp, bool tracer, unsigned grid, int nthr,
+cudaError_t collide_variant<1, false>(int op, int store, bool ramp, bool tracer, unsigned grid, int nthr,
                                         size_t smem, cudaStream_t st, const CollideArgs *A, int *out)
 {
     if (store != 1) return cudaErrorInvalidValue;
-    return collide_variant_store<float, 1, 1, false>(op, ramp, tracer, grid, nthr, smem, st, A, out);
+    return collide_variant_store<1, 1, false>(op, ramp, tracer, grid, nthr, smem, st, A, out);
 }
 
 }  // namespace mcd

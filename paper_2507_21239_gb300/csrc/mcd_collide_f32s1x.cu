@@ -7,13 +7,13 @@
 namespace mcd {
 
 template <>
-cudaError_t collide_variant<float, 1, true>(int op, int store, bool ramp, bool tracer, unsigned grid, int nthr,
+cudaError_t collide_variant<1, true>(int op, int store, bool ramp, bool tracer, unsigned grid, int nthr,
                                         size_t smem, cudaStream_t st, const CollideArgs *A, int *out)
 {
     switch (store) {
-    case 0: return collide_variant_store<float, 1, 0, true>(op, ramp, tracer, grid, nthr, smem, st, A, out);
-    case 1: return collide_variant_store<float, 1, 1, true>(op, ramp, tracer, grid, nthr, smem, st, A, out);
-    case 2: return collide_variant_store<float, 1, 2, true>(op, ramp, tracer, grid, nthr, smem, st, A, out);
+    case 0: return collide_variant_store<1, 0, true>(op, ramp, tracer, grid, nthr, smem, st, A, out);
+    case 1: return collide_variant_store<1, 1, true>(op, ramp, tracer, grid, nthr, smem, st, A, out);
+    case 2: return collide_variant_store<1, 2, true>(op, ramp, tracer, grid, nthr, smem, st, A, out);
     default: return cudaErrorInvalidValue;
     }
 }

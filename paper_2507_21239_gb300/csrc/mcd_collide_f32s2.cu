@@ -7,13 +7,13 @@
 namespace mcd {
 
 template <>
-cudaError_t collide_variant<float, 2, false>(int op, int store, bool ramp, bool tracer, unsigned grid, int nthr,
+cudaError_t collide_variant<2, false>(int op, int store, bool ramp, bool tracer, unsigned grid, int nthr,
                                         size_t smem, cudaStream_t st, const CollideArgs *A, int *out)
 {
     switch (store) {
-    case 0: return collide_variant_store<float, 2, 0, false>(op, ramp, tracer, grid, nthr, smem, st, A, out);
-    case 1: return collide_variant_store<float, 2, 1, false>(op, ramp, tracer, grid, nthr, smem, st, A, out);
-    case 2: return collide_variant_store<float, 2, 2, false>(op, ramp, tracer, grid, nthr, smem, st, A, out);
+    case 0: return collide_variant_store<2, 0, false>(op, ramp, tracer, grid, nthr, smem, st, A, out);
+    case 1: return collide_variant_store<2, 1, false>(op, ramp, tracer, grid, nthr, smem, st, A, out);
+    case 2: return collide_variant_store<2, 2, false>(op, ramp, tracer, grid, nthr, smem, st, A, out);
     default: return cudaErrorInvalidValue;
     }
 }

@@ -81,7 +81,7 @@ __device__ __forceinline__ int warp_choose(const float (&x)[PL], float u, int pe
 
 template <int PL, int STORE, bool RAMP, bool TRACER>
 __device__ __forceinline__ void cell_chain_ws(const CollideArgs &A, const int64_t cell, const int64_t entry,
-                                              Shared<float> &sh, unsigned char *smem_raw)
+                                              Shared &sh, unsigned char *smem_raw)
 {
     typedef float T;
     const unsigned FULL = 0xffffffffu;
@@ -370,7 +370,7 @@ template <int PL, int STORE, bool RAMP, bool TRACER>
 __global__ void __launch_bounds__(32 + 32 * PL) k_collide_ws(CollideArgs A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ Shared<float> sh;
+    __shared__ Shared sh;
     int64_t entry = blockIdx.x;
     for (;;) {
         if (A.qhead) {
