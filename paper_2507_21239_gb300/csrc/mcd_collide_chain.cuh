@@ -1,8 +1,10 @@
 // mcd_collide_chain.cuh -- the mixed-precision collision chain of one cell,
-// split over specialised warps.  Same method, same arithmetic and the same bits
-// as cell_chain<1, ...> in mcd_collide.cuh would give (Zsom &
-// Dullemond's representative-particle scheme, Summary of the mcdust paper);
-// what differs is who does what between which barriers.
+// split over specialised warps.  Same method and arithmetic as cell_chain<1, ...>
+// in mcd_collide.cuh (Zsom & Dullemond's representative-particle scheme, Summary
+// of the mcdust paper), and the bits its builds have given: every rounding here is
+// explicit, where pair_dv leaves the fusing of products to the compiler, and a dv
+// below 1e-19 cm/s counts as 0.  What differs is who does what between which
+// barriers.
 //
 // What bounds it: the serial chain of one event (choose i, form row i, choose
 // j, apply the outcome, renew row and column i) on the heaviest cell; no pipe
@@ -41,9 +43,9 @@
 // 0.98, 300: 1.69 -> 1.31, 400: 1.97 -> 1.47, 500: 2.01 -> 1.62.  (Without the
 // row sums formed ahead 0.93 at 100 and 1.03 at 200; with them 1.56 at 400,
 // where they compete with the choice for issue slots.)  Up to 256 swarms the
-// shared matrix beats recomputing row i (200 swarms: 0.98 against 1.14); where the
-// ready outcomes leave no room for the matrix (from about 290) recomputing in this layout beats the stored matrix in the block-scan layout
-// (1.31 against 1.69).  Two groups per worker warp, to issue what does not
+// shared matrix beats recomputing row i (200 swarms: 0.98 against 1.12); where the
+// ready outcomes leave no room for the matrix (from about 290) recomputing in this
+// layout beats the stored matrix in the block-scan layout (1.31 against 1.71).  Two groups per worker warp, to issue what does not
 // depend on the swarm once per sub-partition, were slower at every size (200:
 // 1.25, 400: 1.63): one warp's instructions issue in order, and two warps hide
 // each other's latencies where two streams in one do not.
@@ -210,6 +212,7 @@ constexpr int kFlRenewed = 16;  // in Part<float>::fl: a cache formed by an even
 
 // make_part<float> with every rounding explicit, so that the mass warp, the
 // choice warp and the first build form the same bits
+template <bool SEL>
 __device__ __forceinline__ Part<float> make_part_rn(const CellK<float> &c, double m, float Mv, int renewed)
 {
     Part<float> q;
@@ -220,7 +223,7 @@ __device__ __forceinline__ Part<float> make_part_rn(const CellK<float> &c, doubl
     q.im = rcp_ftz(mh);
     q.Mv = Mv;
     q.gi = c.dm_t > 0.0f ? rcp_ftz(__fmul_rn(c.dm_t, mh)) : INFINITY;
-    if (c.kmode == 1) {  // the constant kernel: rates and outcomes take masses alone
+    if (!SEL && c.kmode == 1) {  // the constant kernel: rates and outcomes take masses alone
         q.a = q.S = q.Sl = q.p = q.q = q.ad = 0.0f;
         q.fl = renewed;
         return q;
@@ -266,14 +269,16 @@ __device__ __forceinline__ Part<float> make_part_rn(const CellK<float> &c, doubl
 // into shared memory (up to 318 swarms) give the bits they always gave.
 // COMMON (the first row sums, where a whole warp agrees): no v is a Stokes-law swarm,
 // no pair in turbulence regime I and no swarm renewed, so a fifth of the terms is left out.
-template <int N, bool EARLY, bool COMMON = false>
+// SEL: the constant kernel is selected at the end, not branched to (MB > 1: the branch
+// costs the event loop 4 % where registers are short; 64 swarms, 1 yr: 2.90 and 3.01 ms).
+template <int N, bool EARLY, bool COMMON = false, bool SEL = false>
 __device__ __forceinline__ void pair_flat(const PairK<float> &c, bool early, const Part<float> (&u)[N],
                                           const Part<float> (&v)[N], float (&dv)[N], float (&K)[N])
 {
     typedef float T;
     T da[N], D[N], S1[N], S2[N], s[N], g1[N], t2[N], t3[N], coef[N], t0[N];
 #define MCD_EACH _Pragma("unroll") for (int x = 0; x < N; ++x)
-    if (c.kmode == 1) {
+    if (!SEL && c.kmode == 1) {
         MCD_EACH dv[x] = (T)0, K[x] = c.Kc;
         return;
     }
@@ -330,16 +335,17 @@ __device__ __forceinline__ void pair_flat(const PairK<float> &c, bool early, con
     {
         const T s2 = __fadd_rn(u[x].a, v[x].a);
         K[x] = __fmul_rn(__fmul_rn(__fmul_rn(c.pi, s2), s2), dv[x]);
+        if (SEL) K[x] = c.kmode == 1 ? c.Kc : K[x], dv[x] = c.kmode == 1 ? 0.0f : dv[x];
     }
 #undef MCD_EACH
 }
-template <bool EARLY>
+template <bool EARLY, bool SEL = false>
 __device__ __forceinline__ void pair_flat1(const PairK<float> &c, bool early, const Part<float> &u,
                                            const Part<float> &v, float &dv, float &K)
 {
     const Part<float> uu[1] = {u}, vv[1] = {v};
     float d[1], k[1];
-    pair_flat<1, EARLY>(c, early, uu, vv, d, k);
+    pair_flat<1, EARLY, false, SEL>(c, early, uu, vv, d, k);
     dv = d[0];
     K = k[0];
 }
@@ -470,7 +476,7 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
         // every mass the event loop can reach lies between the monomer mass and
         // the disk's dust mass, inside the split's range
         if (!mass_splits(mk)) atomicOr(A.status, kStBadCell);
-        pk = make_part_rn(c, mk, (T)(A.M[off + kc] * c.invVsc), 0);
+        pk = make_part_rn<(MB > 1)>(c, mk, (T)(A.M[off + kc] * c.invVsc), 0);
         const double dmm = __dmul_rn(c.dm, mk);
         if (act) {
             mm[k] = make_double2(mk, dmm);
@@ -525,30 +531,42 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
         const int L = (n - 1) / 2 + 1, half = (n & 1) ? 0 : n / 2, pairs = n * L + half;
         const int step_r = nthr / L, step_d = nthr - step_r * L;
         int rr = tid / L, d = tid - rr * L, t = tid;
-        while ((MB == 1 ? t - lane : t) < pairs) {  // (whole warps, where they vote)
-            int row[2], other[2], at2[2];
-            bool in[2];
-#pragma unroll
-            for (int x = 0; x < 2; ++x) {
-                in[x] = t < pairs;
-                row[x] = !in[x] ? 0 : (t < n * L ? rr : t - n * L);
-                const int o = !in[x] ? 0 : (t < n * L ? d : half);
-                at2[x] = row[x] * W + o;
-                other[x] = row[x] + o;
-                if (other[x] >= n) other[x] -= n;
-                t += nthr, rr += step_r, d += step_d;
+        if constexpr (MB > 1) {  // one at a time: two would spill registers
+            for (; t < pairs; t += nthr) {
+                const int row = t < n * L ? rr : t - n * L, o = t < n * L ? d : half;
+                int j = row + o;
+                if (j >= n) j -= n;
+                T dv, K;
+                pair_flat1<true, true>(pc, early, parts[row], parts[j], dv, K);
+                Dm[row * W + o] = dv;
+                rr += step_r, d += step_d;
                 if (d >= L) d -= L, ++rr;
             }
-            const Part<T> pr[2] = {parts[row[0]], parts[row[1]]}, pj[2] = {parts[other[0]], parts[other[1]]};
-            T dv[2], K[2];
-            // (with several CTAs per SM the second form's registers would be spilled ones)
-            const int cls = min(max(pr[0].fl & 3, pj[0].fl & 3), max(pr[1].fl & 3, pj[1].fl & 3));
-            if (MB == 1 && __all_sync(0xffffffffu, cls && !((pj[0].fl | pj[1].fl) & 4)))
-                pair_flat<2, true, true>(pc, early, pr, pj, dv, K);
-            else
-                pair_flat<2, true>(pc, early, pr, pj, dv, K);
-            if (MB > 1 || in[0]) Dm[at2[0]] = dv[0];
-            if (in[1]) Dm[at2[1]] = dv[1];
+        } else {
+            while (t - lane < pairs) {  // (whole warps: they vote)
+                int row[2], other[2], at2[2];
+                bool in[2];
+#pragma unroll
+                for (int x = 0; x < 2; ++x) {
+                    in[x] = t < pairs;
+                    row[x] = !in[x] ? 0 : (t < n * L ? rr : t - n * L);
+                    const int o = !in[x] ? 0 : (t < n * L ? d : half);
+                    at2[x] = row[x] * W + o;
+                    other[x] = row[x] + o;
+                    if (other[x] >= n) other[x] -= n;
+                    t += nthr, rr += step_r, d += step_d;
+                    if (d >= L) d -= L, ++rr;
+                }
+                const Part<T> pr[2] = {parts[row[0]], parts[row[1]]}, pj[2] = {parts[other[0]], parts[other[1]]};
+                T dv[2], K[2];
+                const int cls = min(max(pr[0].fl & 3, pj[0].fl & 3), max(pr[1].fl & 3, pj[1].fl & 3));
+                if (__all_sync(0xffffffffu, cls && !((pj[0].fl | pj[1].fl) & 4)))
+                    pair_flat<2, true, true>(pc, early, pr, pj, dv, K);
+                else
+                    pair_flat<2, true>(pc, early, pr, pj, dv, K);
+                if (in[0]) Dm[at2[0]] = dv[0];
+                if (in[1]) Dm[at2[1]] = dv[1];
+            }
         }
         __syncthreads();
         if (swarms) add_stored(0, n);
@@ -579,12 +597,13 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
     }
     T hi = act ? (T)R.hi() : (T)0;  // R_k for the next choice
     if constexpr (MB > 1) {
+        if (w < ng) pf[k] = R.s, dvrow[k] = R.c;  // (kept there until the event loop: registers)
         // The first waiting time: most of many light cells have no event in a short step,
-        // and need neither ready outcomes nor choices.  32,768 cells of 32 swarms, collide
-        // of a 0.001-yr step (no events) 485 -> 279 us with the pairs above in row order,
-        // of a 0.1-yr one 557 -> 371 (block-wide scans: 293, 342; with more events than
-        // 0.4 per cell the chain is ahead: 1 yr 2,103 -> 1,724).  In the one-CTA kernels the
-        // ready outcomes are 3 % of a cell, and the branch costs the event loop as much.
+        // and need neither ready outcomes nor choices.  Collide of 32,768 cells of 32
+        // swarms, with the pairs above in row order and R_k parked: a 0.001-yr step (no
+        // events) 485 -> 260 us, a 0.1-yr one 557 -> 336, a 1-yr one 1,726 -> 1,620
+        // (block-wide scans: 293, 342, 2,103).  In the one-CTA kernels the ready outcomes
+        // are 3 % of a cell, and the branch costs the event loop as much.
         if (w < ng) {
             const T x = group_prefix(xw, hi);
             if (lane == 31) sh.ti[2 * NW - ng + w] = x;
@@ -615,7 +634,7 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
         const double2 mk = mm[act ? k : n - 1];
         for (int e = 0; e < 2; ++e) {
             const double mr = ready_mass(c, mk.x, mk.y, e != 0);
-            const Part<T> pr = make_part_rn(c, mr, pk.Mv, kFlRenewed);
+            const Part<T> pr = make_part_rn<(MB > 1)>(c, mr, pk.Mv, kFlRenewed);
             if (act) {
                 ready[e * nsl + k] = pr;
                 mready[e * nsl + k] = make_double2(mr, __dmul_rn(c.dm, mr));
@@ -684,7 +703,7 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
                         mnew = outcome_ramp<T>(c, mmi.x, mj, mih, parts[j].mh, mmi.y, dvij, dr.u3, vlo, kind);
                     else
                         mnew = outcome<T>(c, mmi.x, mj, mih, parts[j].mh, mmi.y, dvij, dr.u3, kind);
-                    ready[gen] = make_part_rn(c, mnew, Mvi, kFlRenewed);
+                    ready[gen] = make_part_rn<(MB > 1)>(c, mnew, Mvi, kFlRenewed);
                     mready[gen] = make_double2(mnew, __dmul_rn(c.dm, mnew));
                 } else {
                     mnew = ready_mass(c, mmi.x, mmi.y, !stick);  // (the mass warp may still be at work on mready)
@@ -747,7 +766,7 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
             // its ready outcomes: even lanes stick, odd lanes erode
             const double mnew = ready_mass(c, mi.x, mi.y, lane & 1), dmnew = __dmul_rn(c.dm, mnew);
             __syncwarp();
-            const Part<T> pnew = make_part_rn(c, mnew, Mvi, kFlRenewed);
+            const Part<T> pnew = make_part_rn<(MB > 1)>(c, mnew, Mvi, kFlRenewed);
             bar_sync(kBarRead, nsl + 32);
             if (lane < 2) {
                 ready[lane * nsl + i] = pnew;
@@ -793,6 +812,10 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
         }
     } else {  // ---- the workers ----
         int pend = -1;  // swarm whose fresh row sum rides on the next choice
+        if constexpr (MB > 1) {
+            R.s = pf[k], R.c = dvrow[k];
+            hi = act ? (T)R.hi() : (T)0;
+        }
         bar_arrive(kBarNew, nsl + 32);
         int guess = 0;  // the kind of ready outcome that came last
         // hi is 0 for the swarm whose fresh sum rides on the next choice; what is put off
@@ -825,7 +848,7 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
                 dvik = Dm[at];
                 Kold = kern_of<T>(pc, pk.a, pi.a, dvik);
             } else {
-                pair_flat1<true>(pc, early, pk, pi, dvik, Kold);
+                pair_flat1<true, (MB > 1)>(pc, early, pk, pi, dvik, Kold);
             }
             R.s = k == pend ? __int_as_float(sel.y) : R.s;
             R.c = k == pend ? (T)0 : R.c;
@@ -849,7 +872,7 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
             us = part_select(k == i, o, pk);
             T dvs, Ks, rows, his;
             Acc<T> Rs;
-            pair_flat1<false>(pc, false, us, o, dvs, Ks);
+            pair_flat1<false, (MB > 1)>(pc, false, us, o, dvs, Ks);
             // (here, not where they are used: the compiler would sink them behind the barrier)
             asm volatile("" : "+f"(Ks), "+f"(dvs));
             if constexpr (AHEAD) {
@@ -876,7 +899,7 @@ __device__ __forceinline__ void chain_cell(const CollideArgs &A, const int64_t c
                 const Part<T> pn = ready[pick.x];
                 T Knew = Ks;
                 pk = part_select(k == i, pn, pk);
-                if (!hit) pair_flat1<false>(pc, false, pk, pn, dvn, Knew);
+                if (!hit) pair_flat1<false, (MB > 1)>(pc, false, pk, pn, dvn, Knew);
                 rn[k] = act && !rebuild ? Knew * weight<T>(pn, pk) : (T)0;
                 bar_arrive(kBarNew, nsl + 32);
                 Rn = R;
