@@ -408,10 +408,11 @@ __device__ __forceinline__ float group_prefix(float *xs, float x)
                      __fadd_rn(__fadd_rn(q[-16], q[-20]), __fadd_rn(q[-24], q[-28])));
 }
 
-// Cells of up to 64 swarms run several CTAs per SM: 32,768 light cells of 40 (64)
-// swarms take 0.81 (1.26) ms with five, 1.45 (1.92) ms with the two that fit
-// without a register limit, while a heavy cell's event takes 0.88 us against
-// 0.80; seven resident CTAs spill (1.29 us).
+// Cells of up to 64 swarms run several CTAs per SM: when the number was chosen,
+// 32,768 light cells of 40 (64) swarms took 0.81 (1.26) ms with five (now 0.78, 1.14),
+// 1.45 (1.92) ms with the two that fit without a register limit, while a heavy cell's
+// event took 0.88 us against 0.80; seven spill (1.29 us), six too (48 swarms, 1 yr: 3.63
+// ms against 3.03).
 constexpr int kChainSmallCtas = 5;
 
 // MB: resident CTAs per SM (cells of up to 64 swarms: many light cells run at

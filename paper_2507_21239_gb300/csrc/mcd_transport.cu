@@ -87,8 +87,8 @@ __device__ __forceinline__ double inv_half_pow(double ix, int k)
 // gas is formed from as few divisions, square roots and transcendental
 // functions as it takes: reciprocals of r, Omega, c_s and rho shared by every
 // quantity, slopes that are multiples of 1/2 without pow(), one expm1 or exp for both
-// exponentials of the vertical step, sincospi.  819,200 particles: 0.83 ms ->
-// 0.42 ms.
+// exponentials of the vertical step, sincospi.  819,200 particles: 0.84 ms ->
+// 0.44 ms with both slopes multiples of 1/2, 0.57 with one pow(), 0.69 with two.
 template <bool TABLE>
 __device__ __forceinline__ void transport_fp64(const DiskC<double> &P, GasTab tab, double &r, double &z, double m,
                                                double dt, const U4 &x)
@@ -181,8 +181,10 @@ __device__ __forceinline__ void transport_mixed(const DiskC<float> &P, GasTab ta
 
 // TABLE: some disk has a gas table (the variant without one reads none).
 // One thread per particle slot.  819,200 particles, mixed: 61 us with every
-// parameter converted per particle on the FP64 unit -> 33 us; what is left is
-// the Philox block's 64-bit products, two powf and the IEEE divisions.
+// parameter converted per particle on the FP64 unit -> 33 us; what is left are 927
+// instructions per warp that issue in 64 % of the cycles, no pipe above 43 % (ALU
+// 43, FP64 40, FMA 33, special functions 14): the Philox block's 64-bit products,
+// two powf, the IEEE divisions, the additions to FP64 positions, and loads waited for.
 template <bool MIXED, bool TABLE>
 __global__ void __launch_bounds__(256) k_transport(const DiskC<typename std::conditional<MIXED, float, double>::type> *consts,
                                                    const GasKnot *gas_knots, const int32_t *gas_n,
